@@ -22,6 +22,7 @@
 
 #include <type_traits>
 
+#include "kbc_fix.cuh"
 #include "kbc_ops.h"
 
 namespace kbc {
@@ -1026,6 +1027,37 @@ __device__ __forceinline__ R collide_lean(R (&d)[27], const CollideParams& cp, i
   return gamma;
 }
 
+// compile-time loop over the 27 velocities
+template <int I, int N> struct Unroll {
+  template <typename F> __device__ __forceinline__ static void run(F&& f) {
+    f(std::integral_constant<int, I>{});
+    Unroll<I + 1, N>::run(f);
+  }
+};
+template <int N> struct Unroll<N, N> {
+  template <typename F> __device__ __forceinline__ static void run(F&&) {}
+};
+
+// The fixed-point collision (kbc_fix.cuh) of the shifts d (FP64 or FP32 values), the result in
+// v (to_f64<nonzero(i)>). False when the node is outside the format's range: v is then nothing,
+// and the caller collides in FP64.
+template <typename S>
+__device__ __forceinline__ bool fix_collide(const S (&d)[27], fix::fx (&v)[27],
+                                            const CollideParams& cp, int* guarded,
+                                            double* gamma) {
+  uint32_t top = 0;
+#pragma unroll
+  for (int i = 0; i < 27; ++i) {
+    if constexpr (std::is_same<S, double>::value) v[i] = fix::from_f64(d[i], &top);
+    else v[i] = fix::from_f32(d[i], &top);
+  }
+  if (top >= (std::is_same<S, double>::value ? fix::kTopF64 : fix::kTopF32)) return false;
+  const fix::Relax rx = {cp.beta, cp.inv_beta, cp.with_t, cp.with_q, cp.gamma_mode};
+  bool bad;
+  *gamma = fix::collide(v, rx, guarded, &bad);
+  return !bad;
+}
+
 // The collision of a step kernel on data in the storage's collision unit (REL: relative to
 // W_i, the FP16 codec): the lean form for FP32 arithmetic, product-form equilibrium and
 // natural moments; collide() otherwise.
@@ -1053,6 +1085,18 @@ __device__ __forceinline__ R collide_step(R (&d)[27], const CollideParams& cp, i
     } else {
       return collide_lean<R, REL>(d, cp, guarded, fp64);
     }
+  } else if constexpr (!CENTRAL && !EXACT && !POLY) {
+    // FP64: the fixed-point collision, or this one in FP64 where the node is outside its range
+    fix::fx v[27];
+    double gam;
+    if (fix_collide(d, v, cp, guarded, &gam)) {
+      Unroll<0, 27>::run([&](auto ic) {
+        constexpr int I = decltype(ic)::value;
+        d[I] = fix::to_f64<fix::nonzero(I)>(v[I]);
+      });
+      return gam;
+    }
+    return collide<R, false, false, false>(d, cp, guarded);
   } else {
     if constexpr (REL) {
 #pragma unroll
@@ -1156,24 +1200,12 @@ template <> struct Pattern<MODE_AA_ODD> {
   __host__ __device__ static constexpr int store_plane(int i) { return i; }
 };
 
-// compile-time loop over the 27 velocities
-template <int I, int N> struct Unroll {
-  template <typename F> __device__ __forceinline__ static void run(F&& f) {
-    f(std::integral_constant<int, I>{});
-    Unroll<I + 1, N>::run(f);
-  }
-};
-template <int N> struct Unroll<N, N> {
-  template <typename F> __device__ __forceinline__ static void run(F&&) {}
-};
-
-// FP64 collision of one node whose FP32 <dh|dh> fell under kDenFp64, after the step kernel:
-// loads the node's inputs where the step's pattern keeps them (pull: src, which the step
-// does not write; AA: the node's own slots, which the step left alone), collides them in
-// FP64 (collide<double>, with the oracle's guard) and stores the outputs in the storage type.
-// Returns gamma; *guarded is set when <dh|dh> fell under the FP64 guard.
+// One node loaded, collided in FP64 instructions (collide<double>, with the oracle's guard) and
+// stored, where the step's pattern keeps its inputs and outputs: the form for nodes that the
+// fixed-point collision does not take. The inputs are still there (pull: src, which a step does
+// not write; AA: the node's own slots, which the caller left alone).
 template <typename S, int MODE, bool CENTRAL, bool POLY>
-__device__ __noinline__ float fp64_node_update(const S* src, S* dst, Geo g, uint32_t x,
+__device__ __noinline__ float fp64_node_native(const S* src, S* dst, Geo g, uint32_t x,
                                                uint32_t y, uint32_t z, CollideParams cp,
                                                int* guarded) {
   using C = Codec<S>;
@@ -1197,6 +1229,35 @@ __device__ __noinline__ float fp64_node_update(const S* src, S* dst, Geo g, uint
   return (float)gam;
 }
 
+// The FP64 update of one node (FP64 storage: every step; FP32 storage: the re-collision of a
+// node whose FP32 <dh|dh> fell under kDenFp64) with the fixed-point collision, natural moments
+// and product form. Returns gamma; *guarded is set when <dh|dh> vanished.
+template <typename S, int MODE>
+__device__ __forceinline__ float fix_node_update(const S* src, S* dst, const Geo& g, uint32_t x,
+                                                 uint32_t y, uint32_t z,
+                                                 const CollideParams& cp, int* guarded) {
+  using C = Codec<S>;
+  using Pat = Pattern<MODE>;
+  Nbr nb;
+  nb.init(g, x, y, z);
+  S d[27];
+  Unroll<0, 27>::run([&](auto ic) {
+    constexpr int I = decltype(ic)::value;
+    const S* p = src + (uint64_t)Pat::load_plane(I) * g.P + nb.template at<I, Pat::load_shift>();
+    d[I] = MODE == MODE_PULL ? __ldg(p) : *p;
+  });
+  fix::fx v[27];
+  double gam;
+  if (!fix_collide(d, v, cp, guarded, &gam))
+    return fp64_node_native<S, MODE, false, false>(src, dst, g, x, y, z, cp, guarded);
+  Unroll<0, 27>::run([&](auto ic) {
+    constexpr int I = decltype(ic)::value;
+    dst[(uint64_t)Pat::store_plane(I) * g.P + nb.template at<I, Pat::store_shift>()] =
+        C::from_delta(fix::to_f64<fix::nonzero(I)>(v[I]), I);
+  });
+  return (float)gam;
+}
+
 // ------------------------------------------------------------------ the fused node update
 // Loads f(x, t) of node (x, y, z) by the pattern of MODE, collides, stores f'(x) where
 // f(t+1) expects it. src and dst are the same buffer in the AA modes.
@@ -1208,6 +1269,15 @@ __device__ __forceinline__ void node_update(const S* src, S* dst, const Geo& g, 
   using C = Codec<S>;
   using R = typename C::R;
   using Pat = Pattern<MODE>;
+  if constexpr (std::is_same<S, double>::value && !CENTRAL && !EXACT && !POLY) {
+    int gd = 0;
+    const float gam = fix_node_update<S, MODE>(src, dst, g, x, y, z, cp, &gd);
+    if constexpr (RECORD) {
+      gamma_out[z * g.nxy + y * g.nx + x] = gam;
+      if (gd) atomicAdd(&ctr->guarded, 1ull);
+    }
+    return;
+  }
   Nbr nb;
   nb.init(g, x, y, z);
   R d[27];

@@ -276,25 +276,52 @@ __global__ void __launch_bounds__(128, 3) batch_adj_kernel(const BoxDesc* __rest
 constexpr int kPassThreads = 256;
 constexpr int kPassBlocks = 152;  // one wave: the pass kernels run one block per SM
 
-// the flagged nodes among mask words w = w0, w0 + stride, ...; returns the guard events
+// the flagged nodes among the mask words of warps w0, w0 + stride, ... (32 words a warp);
+// returns the guard events. A warp takes its words' flagged nodes 32 at a time in the node order,
+// a node per lane, so that runs of flagged nodes are read and written coalesced; a node per word
+// and thread (words in a loop over their bits) touched a sector per value and took 20 ms for a
+// full 256^3 box.
 template <typename S, int MODE, bool CENTRAL, bool POLY>
 __device__ unsigned long long fp64_pass_words(const S* src, S* dst, const Geo& g,
                                               const CollideParams& cp,
                                               float* gamma_out, int record, uint32_t w0,
                                               uint32_t stride) {
-  const uint32_t words = (uint32_t)((g.P + 31) >> 5);
+  const uint32_t words = (uint32_t)((g.P + 31) >> 5), lane = threadIdx.x & 31;
   unsigned long long guards = 0;
-  for (uint32_t w = w0; w < words; w += stride) {
-    uint32_t m = g.fbmask[w];
-    if (m == 0) continue;
-    g.fbmask[w] = 0;
-    while (m) {
-      const uint32_t n = 32 * w + (uint32_t)(__ffs(m) - 1);
-      m &= m - 1;
+  for (uint32_t base = 32 * w0; base < words; base += 32 * stride) {
+    const uint32_t w = base + lane;
+    const uint32_t mine = w < words ? g.fbmask[w] : 0;
+    if (!__any_sync(0xffffffffu, mine != 0)) continue;
+    if (mine) g.fbmask[w] = 0;
+    uint32_t end = __popc(mine);  // flagged nodes up to and including this lane's word
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t up = __shfl_up_sync(0xffffffffu, end, o);
+      if (lane >= o) end += up;
+    }
+    const uint32_t total = __shfl_sync(0xffffffffu, end, 31);
+    for (uint32_t k0 = 0; k0 < total; k0 += 32) {
+      const uint32_t k = k0 + lane;
+      uint32_t slot = 0;  // the word that holds the k-th flagged node: the first with end > k
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const uint32_t e = __shfl_sync(0xffffffffu, end, slot + o - 1);
+        if (e <= k) slot += o;
+      }
+      slot = slot > 31 ? 31 : slot;
+      const uint32_t m = __shfl_sync(0xffffffffu, mine, slot);
+      const uint32_t e = __shfl_sync(0xffffffffu, end, slot);
+      if (k >= total) continue;
+      const uint32_t bit = __fns(m, 0, (int)(k - (e - __popc(m))) + 1);
+      const uint32_t n = 32 * (base + slot) + bit;
       const uint32_t z = n / g.nxy, r = n - z * g.nxy;
       const uint32_t y = r / g.nx, x = r - y * g.nx;
       int gd = 0;
-      const float gam = fp64_node_update<S, MODE, CENTRAL, POLY>(src, dst, g, x, y, z, cp, &gd);
+      float gam;
+      if constexpr (!CENTRAL && !POLY)
+        gam = fix_node_update<S, MODE>(src, dst, g, x, y, z, cp, &gd);
+      else
+        gam = fp64_node_native<S, MODE, CENTRAL, POLY>(src, dst, g, x, y, z, cp, &gd);
       if (record) {
         gamma_out[n] = gam;
         guards += (unsigned long long)gd;
@@ -320,8 +347,8 @@ __global__ void __launch_bounds__(kPassThreads) fp64_pass_kernel(const S* src, S
   if (*(volatile unsigned int*)&ctr->fb_any == 0) return;
   const unsigned long long guards =
       fp64_pass_words<S, MODE, CENTRAL, POLY>(src, dst, g, cp, gamma_out, record,
-                                              blockIdx.x * blockDim.x + threadIdx.x,
-                                              gridDim.x * blockDim.x);
+                                              (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+                                              (gridDim.x * blockDim.x) >> 5);
   if (guards) atomicAdd(&ctr->guarded, guards);
   if (pass_last_block(&ctr->fb_done)) {
     ctr->fb_any = 0;
@@ -344,8 +371,8 @@ __global__ void __launch_bounds__(kPassThreads) batch_fp64_pass_kernel(
     S* dst = (S*)bd.pop[MODE == MODE_PULL ? (parity ^ 1) : 0];
     const unsigned long long guards =
         fp64_pass_words<S, MODE, CENTRAL, false>(src, dst, g, cp, bd.gamma, record,
-                                                 blockIdx.x * blockDim.x + threadIdx.x,
-                                                 gridDim.x * blockDim.x);
+                                                 (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+                                                 (gridDim.x * blockDim.x) >> 5);
     if (guards) atomicAdd(&bd.ctr->guarded, guards);
   }
   if (pass_last_block(&flags->done)) {
