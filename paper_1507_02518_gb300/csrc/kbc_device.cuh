@@ -203,7 +203,7 @@ template <> struct Guard<float> { static constexpr float den = 1e-30f; };
 // With FP32 storage, an FP32 collision whose <dh|dh> falls under kDenFp64 is not used: the
 // lane is flagged (*fp64 bit k), the node's bit is set in the box's mask (flag_fp64), and a
 // pass launched after the step kernel (fp64_pass_kernel) collides the node again in FP64
-// from its inputs (fp64_node_update), with the FP64 guard of the oracle. The inputs are still
+// from its inputs (fix_node_update), with the FP64 guard of the oracle. The inputs are still
 // in memory then: the pull step reads src only and stores the flagged node's FP32 outputs
 // anyway (the pass overwrites them), the AA step does not store a flagged node (each AA node
 // alone reads and writes its slots). The step kernels hold no call of the FP64 path, which
@@ -224,6 +224,7 @@ struct CollideParams {
   double two_beta;  // 2 beta
   double inv_beta;  // 1 / beta
   float betaf, two_betaf, inv_betaf;  // the same, rounded once on the host for FP32 kernels
+  fix::fx quarter_beta, two_beta_1;   // the same for the fixed-point collision
   int with_t;       // shear part includes t (Table 1)
   int with_q;       // shear part includes q (Table 1)
   int gamma_mode;   // GAMMA_*
@@ -1052,7 +1053,8 @@ __device__ __forceinline__ bool fix_collide(const S (&d)[27], fix::fx (&v)[27],
     else v[i] = fix::from_f32(d[i], &top);
   }
   if (top >= (std::is_same<S, double>::value ? fix::kTopF64 : fix::kTopF32)) return false;
-  const fix::Relax rx = {cp.beta, cp.inv_beta, cp.with_t, cp.with_q, cp.gamma_mode};
+  const fix::Relax rx = {cp.quarter_beta, cp.two_beta_1, cp.inv_beta,
+                         cp.with_t,       cp.with_q,     cp.gamma_mode};
   bool bad;
   *gamma = fix::collide(v, rx, guarded, &bad);
   return !bad;

@@ -30,6 +30,23 @@ __global__ void __launch_bounds__(MaxThreads<S>::value) step_kernel(const S* src
   node_update<S, MODE, RECORD, CENTRAL, EXACT, POLY>(src, dst, g, x, y, z, cp, gamma_out, ctr);
 }
 
+// The FP64 step with the fixed-point collision, one node per thread over the node order, so that
+// rows of any length keep every lane busy (the two divisions are nothing beside the ~3400
+// instructions of the collision): 100^3 188 us, with 128-thread rows 22 % of the lanes idled.
+// 168 registers give 12 warps per SM; 256^3 pull takes 2.87 ms at 168, 2.83 at 128 (more spills,
+// 32^3 12.3 instead of 10.3 us), 2.92 at 104, 3.5 at 255.
+template <int MODE, bool RECORD>
+__global__ void __maxnreg__(168) fix_step_kernel(const double* src, double* dst, Geo g,
+                                                         CollideParams cp, float* gamma_out,
+                                                         StepCounters* ctr) {
+  const uint32_t n = g.zb * g.nxy + blockIdx.x * blockDim.x + threadIdx.x;  // P < 2^31
+  if (n >= g.ze * g.nxy) return;
+  const uint32_t row = n / g.nx;
+  const uint32_t x = n - row * g.nx;
+  const uint32_t z = row / g.ny;
+  node_update<double, MODE, RECORD>(src, dst, g, x, row - z * g.ny, z, cp, gamma_out, ctr);
+}
+
 // Moves node (x, y, z) of a box with rows of nx nodes and planes of ny rows k nodes forward in
 // the node order (x fastest); x may start at or beyond nx (it is reduced first).
 __device__ __forceinline__ void advance_node(uint32_t& x, uint32_t& y, uint32_t& z, uint32_t k,
@@ -170,6 +187,8 @@ __device__ __forceinline__ CollideParams box_cp(const BoxDesc& bd, int with_t, i
   cp.betaf = (float)bd.beta;
   cp.two_betaf = (float)bd.two_beta;
   cp.inv_betaf = (float)bd.inv_beta;
+  cp.quarter_beta = bd.quarter_beta;
+  cp.two_beta_1 = bd.two_beta_1;
   cp.with_t = with_t;
   cp.with_q = with_q;
   cp.gamma_mode = gamma_mode;
@@ -269,12 +288,12 @@ __global__ void __launch_bounds__(128, 3) batch_adj_kernel(const BoxDesc* __rest
 // ------------------------------------------------------------------ FP64 re-collision pass
 // A step kernel (FP32 storage) that meets a node whose FP32 <dh|dh> fell under kDenFp64 sets
 // its bit in the box's mask (flag_fp64) and, in AA, does not store it. The pass launched
-// after it collides every flagged node again in FP64 from its inputs (fp64_node_update) and
+// after it collides every flagged node again in FP64 from its inputs (fix_node_update) and
 // clears the mask. When nothing was flagged (the usual case) it
 // reads one flag and exits. The last of its blocks to finish clears the flags; all blocks
 // have read them by then.
-constexpr int kPassThreads = 256;
-constexpr int kPassBlocks = 152;  // one wave: the pass kernels run one block per SM
+constexpr int kPassThreads = 384;  // 12 warps at 168 registers
+constexpr int kPassBlocks = 152;   // one wave: the pass kernels run one block per SM
 
 // the flagged nodes among the mask words of warps w0, w0 + stride, ... (32 words a warp);
 // returns the guard events. A warp takes its words' flagged nodes 32 at a time in the node order,
@@ -406,6 +425,8 @@ inline CollideParams make_cp(double beta, int with_t, int with_q, int gamma_mode
   cp.betaf = (float)cp.beta;
   cp.two_betaf = (float)cp.two_beta;
   cp.inv_betaf = (float)cp.inv_beta;
+  cp.quarter_beta = fix::quarter_beta(beta);
+  cp.two_beta_1 = fix::two_beta_1(beta);
   cp.with_t = with_t;
   cp.with_q = with_q;
   cp.gamma_mode = gamma_mode;
@@ -452,6 +473,13 @@ static cudaError_t launch_step_c(const BoxView& b, const S* src, S* dst, const G
     if (o.kernel == KERNEL_PACKED || o.kernel == KERNEL_AUTO || o.kernel == KERNEL_ROWS)
       return launch_pair<S, MODE, RECORD, CENTRAL, POLY>(src, dst, g, cp, b.gamma, ctr, st);
   }
+  if constexpr (std::is_same<S, double>::value && !CENTRAL && !POLY) {
+    const uint32_t threads = o.bx * o.by;
+    const uint32_t nodes = (g.ze - g.zb) * g.nxy;
+    fix_step_kernel<MODE, RECORD><<<(nodes + threads - 1) / threads, threads, 0, st>>>(
+        src, dst, g, cp, b.gamma, ctr);
+    return cudaGetLastError();
+  }
   const dim3 block(o.bx, o.by, 1);
   const dim3 grid((b.nx + o.bx - 1) / o.bx, (b.ny + o.by - 1) / o.by, g.ze - g.zb);
   step_kernel<S, MODE, RECORD, CENTRAL, false, POLY><<<grid, block, 0, st>>>(src, dst, g, cp,
@@ -468,8 +496,8 @@ static cudaError_t launch_step_p(const BoxView& b, const S* src, S* dst, const G
   cudaError_t e = launch_step_c<S, MODE, RECORD, CENTRAL, POLY>(b, src, dst, g, cp, o, ctr, st);
   if constexpr (std::is_same<S, float>::value) {
     if (e == cudaSuccess && cp.gamma_mode == GAMMA_ESTIMATE) {
-      const uint64_t words = (g.P + 31) / 32;
-      uint64_t blocks = (words + kPassThreads - 1) / kPassThreads;
+      const uint64_t warps = (g.P + 1023) / 1024;  // a warp takes 32 mask words
+      uint64_t blocks = (32 * warps + kPassThreads - 1) / kPassThreads;
       if (blocks > (uint64_t)kPassBlocks) blocks = kPassBlocks;
       fp64_pass_kernel<S, MODE, CENTRAL, POLY><<<(unsigned)blocks, kPassThreads, 0, st>>>(
           src, dst, g, cp, b.gamma, ctr, RECORD ? 1 : 0);

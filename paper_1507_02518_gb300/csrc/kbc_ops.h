@@ -74,6 +74,7 @@ struct BoxDesc {
   uint32_t* fbmask;
   StepCounters* ctr;
   double beta, two_beta, inv_beta;
+  long long quarter_beta, two_beta_1;  // beta / 4 of 2^64 and 2 beta - 1 of 2^62 (kbc_fix.cuh)
 };
 
 template <typename S> struct Ops {

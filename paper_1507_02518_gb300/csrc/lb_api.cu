@@ -15,6 +15,7 @@
 #include <utility>
 #include <vector>
 
+#include "kbc_fix.cuh"
 #include "kbc_lb.h"
 #include "kbc_ops.h"
 
@@ -1502,6 +1503,8 @@ lb_status lb_batch_create(const lb_config* cfgs, int32_t nbox, void* dev_buf, si
       d.beta = v->box.beta;
       d.two_beta = 2.0 * v->box.beta;
       d.inv_beta = 1.0 / v->box.beta;
+      d.quarter_beta = kbc::fix::quarter_beta(v->box.beta);
+      d.two_beta_1 = kbc::fix::two_beta_1(v->box.beta);
     }
     e = cudaMemcpyAsync(b->d_boxes, descs.data(), sizeof(kbc::BoxDesc) * nbox,
                         cudaMemcpyHostToDevice, b->stream);

@@ -21,7 +21,8 @@ WRAP = r'''
 using namespace kbc;
 extern "C" void fix_collide(int n, const double* d, double* o, double* g, int* flags, double beta,
                             int wt, int wq, int mode) {
-  fix::Relax rx = {beta, 1.0 / beta, wt, wq, mode};
+  const fix::Relax rx = {fix::quarter_beta(beta), fix::two_beta_1(beta), 1.0 / beta,
+                         wt, wq, mode};
   for (int k = 0; k < n; ++k) {
     fix::fx v[27];
     uint32_t top = 0;
@@ -146,6 +147,20 @@ def test_error_is_not_above_that_of_fp64(lib, shear, higher, wt, wq, mode):
 def test_rest_is_guarded_and_kept(lib):
     o, g, fl = collide(lib, np.zeros((1, 27)), 0.9, 1, 1, 0)
     assert fl[0] == 1 and g[0] == 2.0 and not o.any()
+
+
+@pytest.mark.parametrize("wt,wq", [(0, 0), (1, 1)])
+def test_equilibrium_states_stay(lib, wt, wq):
+    """Deviations of a unit or none: gamma is a ratio of nothing, the node must not move."""
+    rng = np.random.default_rng(9)
+    u = rng.uniform(-0.1, 0.1, (3, 3000)) * rng.integers(0, 2, (3, 3000))
+    d = (product_equilibrium(np.ones(3000, dtype=LD), u.astype(LD), LD) - weights(LD))
+    d = d.astype(np.float64)
+    o, _, fl = collide(lib, d, 0.99, wt, wq, 0)
+    ok = (fl & 2) == 0
+    assert ok.mean() > 0.9 and (fl & 1).any()
+    # |f' - f| is bounded by the deviations (a few units each, 27 of them) whatever gamma is
+    assert np.abs(o - d)[ok].max() <= 1000 * 2.0 ** -60
 
 
 @pytest.mark.parametrize("what", ["nan", "inf", "shift", "rho", "u", "gamma"])
