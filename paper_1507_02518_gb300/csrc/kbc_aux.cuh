@@ -29,91 +29,299 @@ __device__ __forceinline__ void node_coords(const Geo& g, uint64_t n, uint32_t& 
   x = r - y * g.nx;
 }
 
-template <typename S>
-__global__ void init_kernel(S* b0, S* b1, Geo g, int scheme, int parity, const double* rho,
-                            const double* u, uint64_t n0, uint64_t cnt, uint64_t ld) {
-  for (uint64_t k = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; k < cnt;
-       k += (uint64_t)gridDim.x * blockDim.x) {
-    uint32_t x, y, z;
-    node_coords(g, n0 + k, x, y, z);
-    Nbr nb;
-    nb.init(g, x, y, z);
-    double dq[27];
-    equilibrium_shift<double>(rho ? rho[k] : 1.0, u[k], u[ld + k], u[2 * ld + k], dq);
-#pragma unroll
-    for (int i = 0; i < 27; ++i)
-      *canon_addr<S>(b0, b1, g, nb, scheme, parity, i) = Codec<S>::from_delta(dq[i], i);
+// The same address for a compile-time layout: KIND 0 pull (buf = the buffer of parity t), 1 AA
+// at even t, 2 AA at odd t (buf = the one AA buffer).
+template <int KIND, int I, typename S>
+__device__ __forceinline__ S* canon_ptr(S* buf, const Geo& g, const Nbr& nb) {
+  if constexpr (KIND == 1) return buf + (uint64_t)I * g.P + nb.template at<I, 0>();
+  else if constexpr (KIND == 0) return buf + (uint64_t)I * g.P + nb.template at<I, -1>();
+  else return buf + (uint64_t)(26 - I) * g.P + nb.template at<I, -1>();
+}
+
+// ------------------------------------------------------------------ transfers
+// The kernels between the stored shifts and the caller's FP64 fields. What they compute is a few
+// operations per population, but GB300 converts to and from FP64 at the rate of its FP64 pipe (2
+// lanes per SM and cycle): with a conversion and an addition there per population they ran at
+// 2 to 15 times the time of their memory traffic. So the conversions are integer operations (a
+// rebiased exponent), sums are integer sums and initial equilibria are computed in fixed point;
+// the one FP64 operation left per population of get and set is the addition or subtraction of
+// W. Values outside the normal ranges go to the compiler's conversions.
+
+// 256^3, FP32 pull, one thread per node (before: a grid-stride loop with the layout picked at run
+// time): get 1.83 -> 1.07 ms, set 1.65 -> 1.33, moments 4.05 -> 0.73, init 6.09 -> 1.01; their
+// traffic alone takes 0.81, 0.81, 0.35, 0.33 ms. FP16: get 1.77 -> 1.06, set 2.52 -> 1.11, moments
+// 4.06 -> 0.62, init 6.98 -> 1.08; FP64: get 1.29 -> 1.08, set 1.55 -> 1.11, moments 3.21 -> 0.76.
+// Moments and init are bound by the integer pipe (400 and 1250 instructions a node), get and set
+// by DRAM and the FP64 addition together.
+
+// FP32 to FP64 exactly for normal numbers; *odd is set for zero, subnormals, infinities and NaN
+__device__ __forceinline__ double widen(float v, bool* odd) {
+  const uint32_t b = __float_as_uint(v), a = b & 0x7fffffffu;
+  *odd |= a - 0x00800000u >= 0x7f000000u;
+  return __hiloint2double((int)((b & 0x80000000u) | ((a >> 3) + 0x38000000u)), (int)(b << 29));
+}
+
+// FP64 to FP32, rounded to nearest even, for results in the normal range below 2^64; *odd is set
+// otherwise (zero too)
+__device__ __forceinline__ float narrow(double v, bool* odd) {
+  const uint32_t h = (uint32_t)__double2hiint(v), l = (uint32_t)__double2loint(v);
+  const uint32_t a = h & 0x7fffffffu;
+  *odd |= a - 0x38100000u >= 0x43f00000u - 0x38100000u;
+  const uint32_t t = __funnelshift_l(l, a - 0x38000000u, 3);
+  const uint32_t rest = l << 3;  // the 29 bits below the result's last
+  const uint32_t r = t + (rest > 0x80000000u - (t & 1u) ? 1u : 0u);
+  return __uint_as_float((h & 0x80000000u) | r);
+}
+
+// f_I = W_I + (stored value), and back, in FP64
+template <typename S, int I> __device__ __forceinline__ double population_of(S v, bool* odd) {
+  if constexpr (std::is_same<S, double>::value) return __dadd_rn(wgt(I), v);
+  else if constexpr (std::is_same<S, float>::value) return __dadd_rn(wgt(I), widen(v, odd));
+  else return __fma_rn(wgt(I), widen(__half2float(__ushort_as_half(v)), odd), wgt(I));
+}
+template <typename S, int I> __device__ __forceinline__ S stored_of(double f, bool* odd) {
+  if constexpr (std::is_same<S, double>::value) {
+    return __dadd_rn(f, -wgt(I));
+  } else if constexpr (std::is_same<S, float>::value) {
+    return narrow(__dadd_rn(f, -wgt(I)), odd);
+  } else {
+    // (f - W) / W in one rounding, to FP32 towards zero with the lost bits in the last one
+    // (round to odd), so that the rounding to half is the only one
+    const double d = __fma_rn(f, inv_wgt(I), -1.0);
+    const uint32_t h = (uint32_t)__double2hiint(d), l = (uint32_t)__double2loint(d);
+    const uint32_t a = h & 0x7fffffffu;
+    *odd |= a - 0x38100000u >= 0x43f00000u - 0x38100000u;
+    const uint32_t t = __funnelshift_l(l, a - 0x38000000u, 3) | ((l << 3) != 0 ? 1u : 0u);
+    return __half_as_ushort(__float2half_rn(__uint_as_float((h & 0x80000000u) | t)));
   }
 }
 
-template <typename S>
-__global__ void get_kernel(const S* b0, const S* b1, Geo g, int scheme, int parity, double* out,
-                           uint64_t n0, uint64_t cnt, uint64_t ld) {
-  for (uint64_t k = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; k < cnt;
-       k += (uint64_t)gridDim.x * blockDim.x) {
-    uint32_t x, y, z;
-    node_coords(g, n0 + k, x, y, z);
-    Nbr nb;
-    nb.init(g, x, y, z);
-#pragma unroll
-    for (int i = 0; i < 27; ++i) {
-      const S v = *canon_addr<S>((S*)b0, (S*)b1, g, nb, scheme, parity, i);
-      out[i * ld + k] = wgt(i) + Codec<S>::to_delta(v, i);
-    }
+template <typename S, int KIND>
+__global__ void __launch_bounds__(256) get_kernel(const S* buf, Geo g, double* out, uint64_t n0,
+                                                  uint64_t cnt, uint64_t ld) {
+  const uint64_t k = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+  if (k >= cnt) return;
+  uint32_t x, y, z;
+  node_coords(g, n0 + k, x, y, z);
+  Nbr nb;
+  nb.init(g, x, y, z);
+  S v[27];
+  Unroll<0, 27>::run([&](auto ic) {
+    constexpr int I = decltype(ic)::value;
+    v[I] = *canon_ptr<KIND, I>(buf, g, nb);
+  });
+  bool odd = false;
+  double f[27];
+  Unroll<0, 27>::run([&](auto ic) {
+    constexpr int I = decltype(ic)::value;
+    f[I] = population_of<S, I>(v[I], &odd);
+  });
+  if (odd) {
+    Unroll<0, 27>::run([&](auto ic) {
+      constexpr int I = decltype(ic)::value;
+      f[I] = wgt(I) + Codec<S>::to_delta(v[I], I);
+    });
   }
+#pragma unroll
+  for (int i = 0; i < 27; ++i) out[i * ld + k] = f[i];
 }
 
-template <typename S>
-__global__ void set_kernel(S* b0, S* b1, Geo g, int scheme, int parity, const double* in,
-                           uint64_t n0, uint64_t cnt, uint64_t ld) {
-  for (uint64_t k = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; k < cnt;
-       k += (uint64_t)gridDim.x * blockDim.x) {
-    uint32_t x, y, z;
-    node_coords(g, n0 + k, x, y, z);
-    Nbr nb;
-    nb.init(g, x, y, z);
+template <typename S, int KIND>
+__global__ void __launch_bounds__(256) set_kernel(S* buf, Geo g, const double* in, uint64_t n0,
+                                                  uint64_t cnt, uint64_t ld) {
+  const uint64_t k = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+  if (k >= cnt) return;
+  uint32_t x, y, z;
+  node_coords(g, n0 + k, x, y, z);
+  Nbr nb;
+  nb.init(g, x, y, z);
+  double f[27];
 #pragma unroll
-    for (int i = 0; i < 27; ++i)
-      *canon_addr<S>(b0, b1, g, nb, scheme, parity, i) =
-          Codec<S>::from_delta(in[i * ld + k] - wgt(i), i);
+  for (int i = 0; i < 27; ++i) f[i] = in[i * ld + k];
+  bool odd = false;
+  S v[27];
+  Unroll<0, 27>::run([&](auto ic) {
+    constexpr int I = decltype(ic)::value;
+    v[I] = stored_of<S, I>(f[I], &odd);
+  });
+  if (odd) {
+    Unroll<0, 27>::run([&](auto ic) {
+      constexpr int I = decltype(ic)::value;
+      v[I] = Codec<S>::from_delta(f[I] - wgt(I), I);
+    });
   }
+  Unroll<0, 27>::run([&](auto ic) {
+    constexpr int I = decltype(ic)::value;
+    *canon_ptr<KIND, I>(buf, g, nb) = v[I];
+  });
 }
 
-// rho and rho u of canonical f(t) at one node, accumulated in FP64 from the shifts
-template <typename S>
-__device__ __forceinline__ void node_moments(const S* b0, const S* b1, const Geo& g,
-                                             const Nbr& nb, int scheme, int parity, double& rho,
-                                             double (&m)[3]) {
+// rho - 1 and rho u of 27 shifts in FP64 arithmetic
+template <typename T>
+__device__ __forceinline__ void moments_fp64(const T (&d)[27], double& drho, double (&m)[3]) {
   double s = 0.0, mx = 0.0, my = 0.0, mz = 0.0;
 #pragma unroll
   for (int i = 0; i < 27; ++i) {
-    const double dv = Codec<S>::to_delta(*canon_addr<S>((S*)b0, (S*)b1, g, nb, scheme, parity, i), i);
+    const double dv = (double)d[i];
     s += dv;
     if (cx(i)) mx += cx(i) * dv;
     if (cy(i)) my += cy(i) * dv;
     if (cz(i)) mz += cz(i) * dv;
   }
-  rho = 1.0 + s;
+  drho = s;
   m[0] = mx;
   m[1] = my;
   m[2] = mz;
 }
 
-template <typename S>
-__global__ void moments_kernel(const S* b0, const S* b1, Geo g, int scheme, int parity,
-                               double* rho_out, double* u_out, uint64_t n0, uint64_t cnt,
-                               uint64_t ld) {
-  for (uint64_t k = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; k < cnt;
-       k += (uint64_t)gridDim.x * blockDim.x) {
-    uint32_t x, y, z;
-    node_coords(g, n0 + k, x, y, z);
-    Nbr nb;
-    nb.init(g, x, y, z);
-    double rho, m[3];
-    node_moments<S>(b0, b1, g, nb, scheme, parity, rho, m);
-    if (rho_out) rho_out[k] = rho;
-    for (int a = 0; a < 3; ++a) u_out[a * ld + k] = m[a] / rho;
+// rho and u of canonical f(t). The shifts of a node are scaled to integers by the node's largest
+// exponent (57 bits below it, so the sums are at least as exact as FP64 sums), summed, and the
+// four sums converted; u is rho u times the reciprocal of rho. FP16: the shifts times 216 are
+// exact FP32 numbers (the weights are 64 : 16 : 4 : 1).
+template <typename S, int KIND>
+__global__ void __launch_bounds__(256) moments_kernel(const S* buf, Geo g, double* rho_out,
+                                                      double* u_out, uint64_t n0, uint64_t cnt,
+                                                      uint64_t ld) {
+  using T = typename std::conditional<std::is_same<S, double>::value, double, float>::type;
+  constexpr bool kHalf = std::is_same<S, uint16_t>::value;
+  constexpr int kMant = std::is_same<T, double>::value ? 52 : 23;
+  constexpr int kBias = std::is_same<T, double>::value ? 1023 : 127;
+  const uint64_t k = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+  if (k >= cnt) return;
+  uint32_t x, y, z;
+  node_coords(g, n0 + k, x, y, z);
+  Nbr nb;
+  nb.init(g, x, y, z);
+  T d[27];
+  uint32_t top = 0;  // the largest sign-free high word
+  Unroll<0, 27>::run([&](auto ic) {
+    constexpr int I = decltype(ic)::value;
+    const S v = *canon_ptr<KIND, I>(buf, g, nb);
+    if constexpr (kHalf)
+      d[I] = __fmul_rn(__half2float(__ushort_as_half(v)), (float)(216.0 * wgt(I)));
+    else
+      d[I] = v;
+  });
+#pragma unroll
+  for (int i = 0; i < 27; ++i) {
+    const uint32_t a = (uint32_t)(fix::bits_of(d[i]) >> (sizeof(T) == 8 ? 32 : 0)) & 0x7fffffffu;
+    top = a > top ? a : top;
   }
+  constexpr int kShift = sizeof(T) == 8 ? 20 : 23;
+  const int et = (int)(top >> kShift);  // biased exponent of the largest
+  double drho, m[3], ir;
+  // the fast path: the largest value between 2^-100 and 1/4 (FP16: 54), rho within the range of
+  // the fixed-point reciprocal
+  bool fast = et > kBias - 100 && et < kBias - 2 + (kHalf ? 8 : 0);
+  if (fast) {
+    fix::fx v[27];
+#pragma unroll
+    for (int i = 0; i < 27; ++i) {
+      const auto b = fix::bits_of(d[i]);
+      const uint32_t h = (uint32_t)(b >> (sizeof(T) == 8 ? 32 : 0));
+      const uint32_t e = (h >> kShift) & (sizeof(T) == 8 ? 0x7ffu : 0xffu);
+      // 1.mantissa with its leading bit at 63, shifted so that the largest has it at 57
+      const uint64_t q = ((uint64_t)b << (63 - kMant)) | 0x8000000000000000ull;
+      const fix::fx a = (fix::fx)fix::shr(e == 0 ? 0 : q, (uint32_t)et + 6u - e);
+      v[i] = (int32_t)h < 0 ? -a : a;
+    }
+    // the four sums, x first
+    fix::fx X0[9], X1[9];
+#pragma unroll
+    for (int r = 0; r < 9; ++r) {
+      X0[r] = v[3 * r] + v[3 * r + 1] + v[3 * r + 2];
+      X1[r] = v[3 * r + 2] - v[3 * r];
+    }
+    const fix::fx zm = X0[0] + X0[1] + X0[2], z0 = X0[3] + X0[4] + X0[5],
+                  zp = X0[6] + X0[7] + X0[8];
+    const fix::fx sum[4] = {zm + z0 + zp,
+                            X1[0] + X1[1] + X1[2] + X1[3] + X1[4] + X1[5] + X1[6] + X1[7] + X1[8],
+                            X0[2] + X0[5] + X0[8] - X0[0] - X0[3] - X0[6], zp - zm};
+    // value = sum 2^(et - bias - 57)
+    const int ex = et - kBias - 57;
+    double val[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const double c = (double)sum[j];
+      const int h = __double2hiint(c);
+      val[j] = __hiloint2double(h == 0 ? 0 : h + ex * (1 << 20), __double2loint(c));
+    }
+    drho = val[0];
+    if constexpr (kHalf) drho *= 1.0 / 216.0;
+    // rho in units of 2^-60 (FP16: 216 rho in units of 2^-52)
+    const int sh = ex + (kHalf ? 52 : 60);
+    const fix::fx ds = sh >= 0 ? fix::shl(sum[0], sh) : (sh < -63 ? 0 : sum[0] >> -sh);
+    const fix::fx r = kHalf ? (216ll << 52) + ds : fix::kOne + ds;
+    fast = r > fix::kOne / 2 && r < 2 * fix::kOne;
+    if (fast) {
+      // 1 / rho, or 1 / (216 rho) = 2^-8 / (r 2^-60)
+      ir = fix::to_f64<kHalf ? 8 : 0>(fix::reciprocal(r));
+#pragma unroll
+      for (int a = 0; a < 3; ++a) m[a] = __dmul_rn(val[a + 1], ir);
+    }
+  }
+  if (!fast) {
+    moments_fp64(d, drho, m);
+    if constexpr (kHalf) {
+      drho /= 216.0;
+      for (int a = 0; a < 3; ++a) m[a] /= 216.0;
+    }
+    for (int a = 0; a < 3; ++a) m[a] /= 1.0 + drho;
+  }
+  if (rho_out) rho_out[k] = 1.0 + drho;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) u_out[a * ld + k] = m[a];
+}
+
+// f_eq(rho, u) in FP64 instructions, stored (FP64 storage, and nodes off the fixed-point range)
+template <typename S, int KIND>
+__device__ __noinline__ void init_node_fp64(S* buf, Geo g, uint32_t x, uint32_t y, uint32_t z,
+                                            double rho, double ux, double uy, double uz) {
+  Nbr nb;
+  nb.init(g, x, y, z);
+  double dq[27];
+  equilibrium_shift<double>(rho, ux, uy, uz, dq);
+  Unroll<0, 27>::run([&](auto ic) {
+    constexpr int I = decltype(ic)::value;
+    *canon_ptr<KIND, I>(buf, g, nb) = Codec<S>::from_delta(dq[I], I);
+  });
+}
+
+// f = f_eq(rho, u). FP32 and FP16 storage: the equilibrium's moments and populations in fixed
+// point (kbc_fix.cuh; 2^-59 absolute, far below the rounding of the stored values), for nodes
+// whose velocity or density shift is at least 2^-18, so that this holds relative to the node too.
+template <typename S, int KIND>
+__global__ void __launch_bounds__(256) init_kernel(S* buf, Geo g, const double* rho,
+                                                   const double* u, uint64_t n0, uint64_t cnt,
+                                                   uint64_t ld) {
+  const uint64_t k = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+  if (k >= cnt) return;
+  uint32_t x, y, z;
+  node_coords(g, n0 + k, x, y, z);
+  const double r = rho ? rho[k] : 1.0, ux = u[k], uy = u[ld + k], uz = u[2 * ld + k];
+  if constexpr (!std::is_same<S, double>::value) {
+    const double dr = r - 1.0;
+    uint32_t top = 0;
+    const fix::fx v[4] = {fix::from_f64(dr, &top), fix::from_f64(ux, &top),
+                          fix::from_f64(uy, &top), fix::from_f64(uz, &top)};
+    if (top < fix::kTopF64 && top >= 0x3ed00000u) {
+      fix::fx p[27];
+      fix::equilibrium(v[0], v[1], v[2], v[3], p);
+      Nbr nb;
+      nb.init(g, x, y, z);
+      Unroll<0, 27>::run([&](auto ic) {
+        constexpr int I = decltype(ic)::value;
+        constexpr int N = fix::nonzero(I);
+        S* q = canon_ptr<KIND, I>(buf, g, nb);
+        if constexpr (std::is_same<S, float>::value)
+          *q = fix::to_f32<N>(p[I]);
+        else  // (f - W) / W = 27/8 4^N (f - W)
+          *q = __half_as_ushort(__float2half_rn(fix::to_f32_odd<3 - N>(27 * p[I])));
+      });
+      return;
+    }
+  }
+  init_node_fp64<S, KIND>(buf, g, x, y, z, r, ux, uy, uz);
 }
 
 // ------------------------------------------------------------------ diagnostics
@@ -141,15 +349,6 @@ __device__ __forceinline__ void block_reduce_store(double (&v)[N], double* dst) 
     for (int w = 0; w < nw; ++w) acc += sh[w][threadIdx.x];
     dst[threadIdx.x] = acc;
   }
-}
-
-// Address of canonical f_I(node, t) for a compile-time layout: KIND 0 pull (buf = the buffer
-// of parity t), 1 AA at even t, 2 AA at odd t (buf = the one AA buffer).
-template <int KIND, int I, typename S>
-__device__ __forceinline__ const S* canon_ptr(const S* buf, const Geo& g, const Nbr& nb) {
-  if constexpr (KIND == 1) return buf + (uint64_t)I * g.P + nb.template at<I, 0>();
-  else if constexpr (KIND == 0) return buf + (uint64_t)I * g.P + nb.template at<I, -1>();
-  else return buf + (uint64_t)(26 - I) * g.P + nb.template at<I, -1>();
 }
 
 // rho - 1 and rho u of canonical f(t) at one node, in the arithmetic type of the storage
@@ -465,38 +664,51 @@ __global__ void convert_u_kernel(const double* u, R* ufield, uint64_t n0, uint64
   }
 }
 
+// launch<KIND>(buffer) for the layout of a box at time t
+template <typename S, typename F>
+static cudaError_t with_layout(const BoxView& b, int64_t t, F&& launch) {
+  const int parity = (int)(t & 1);
+  if (b.scheme == 0) launch(std::integral_constant<int, 0>{}, (S*)b.pop[parity]);
+  else if (parity == 0) launch(std::integral_constant<int, 1>{}, (S*)b.pop[0]);
+  else launch(std::integral_constant<int, 2>{}, (S*)b.pop[0]);
+  return cudaGetLastError();
+}
+inline unsigned node_blocks(uint64_t cnt) { return (unsigned)((cnt + 255) / 256); }
+
 template <typename S>
 cudaError_t Ops<S>::init(const BoxView& b, int64_t t, const double* rho, const double* u,
                          uint64_t n0, uint64_t cnt, uint64_t ld, cudaStream_t st) {
-  init_kernel<S><<<grid_for(cnt, 256), 256, 0, st>>>((S*)b.pop[0], (S*)b.pop[1], make_geo(b),
-                                                     b.scheme, (int)(t & 1), rho, u, n0, cnt, ld);
-  return cudaGetLastError();
+  return with_layout<S>(b, t, [&](auto kind, S* buf) {
+    init_kernel<S, decltype(kind)::value><<<node_blocks(cnt), 256, 0, st>>>(
+        buf, make_geo(b), rho, u, n0, cnt, ld);
+  });
 }
 
 template <typename S>
 cudaError_t Ops<S>::get(const BoxView& b, int64_t t, double* out, uint64_t n0, uint64_t cnt,
                         uint64_t ld, cudaStream_t st) {
-  get_kernel<S><<<grid_for(cnt, 256), 256, 0, st>>>((const S*)b.pop[0], (const S*)b.pop[1],
-                                                    make_geo(b), b.scheme, (int)(t & 1), out, n0,
-                                                    cnt, ld);
-  return cudaGetLastError();
+  return with_layout<S>(b, t, [&](auto kind, S* buf) {
+    get_kernel<S, decltype(kind)::value><<<node_blocks(cnt), 256, 0, st>>>(buf, make_geo(b), out,
+                                                                           n0, cnt, ld);
+  });
 }
 
 template <typename S>
 cudaError_t Ops<S>::set(const BoxView& b, int64_t t, const double* in, uint64_t n0,
                         uint64_t cnt, uint64_t ld, cudaStream_t st) {
-  set_kernel<S><<<grid_for(cnt, 256), 256, 0, st>>>((S*)b.pop[0], (S*)b.pop[1], make_geo(b),
-                                                    b.scheme, (int)(t & 1), in, n0, cnt, ld);
-  return cudaGetLastError();
+  return with_layout<S>(b, t, [&](auto kind, S* buf) {
+    set_kernel<S, decltype(kind)::value><<<node_blocks(cnt), 256, 0, st>>>(buf, make_geo(b), in,
+                                                                           n0, cnt, ld);
+  });
 }
 
 template <typename S>
 cudaError_t Ops<S>::moments(const BoxView& b, int64_t t, double* rho, double* u, uint64_t n0,
                             uint64_t cnt, uint64_t ld, cudaStream_t st) {
-  moments_kernel<S><<<grid_for(cnt, 256), 256, 0, st>>>((const S*)b.pop[0], (const S*)b.pop[1],
-                                                        make_geo(b), b.scheme, (int)(t & 1), rho,
-                                                        u, n0, cnt, ld);
-  return cudaGetLastError();
+  return with_layout<S>(b, t, [&](auto kind, S* buf) {
+    moments_kernel<S, decltype(kind)::value><<<node_blocks(cnt), 256, 0, st>>>(
+        buf, make_geo(b), rho, u, n0, cnt, ld);
+  });
 }
 
 template <typename S>

@@ -167,6 +167,29 @@ template <int N> KBC_HD double to_f64(fx v) {
   return f64_of((uint64_t)hi << 32 | (uint32_t)b);
 }
 
+// v * 2^-(60 + n) in FP32: rounded to nearest even, or towards zero with the lost bits in the
+// last one (round to odd: a further rounding to a shorter type is then the only one)
+KBC_HD float i2f(uint32_t x) { return (float)x; }
+template <int N> KBC_HD float to_f32(fx v) {
+  const uint64_t a = v < 0 ? 0 - (uint64_t)v : (uint64_t)v;
+  const int lz = clz64(a);
+  const uint64_t q = lz == 64 ? 0 : a << lz;
+  // the leading 32 bits, the rest as a sticky bit: the conversion rounds at bit 24
+  const uint32_t t = (uint32_t)(q >> 32) | ((uint32_t)q != 0 ? 1u : 0u);
+  const uint32_t b = bits_of(i2f(t));  // t 2^(32 - lz) of the units
+  const uint32_t r = t == 0 ? 0 : b + ((uint32_t)(32 - kFrac - N - lz) << 23);
+  return f32_of(r | ((uint32_t)((uint64_t)v >> 32) & 0x80000000u));
+}
+template <int N> KBC_HD float to_f32_odd(fx v) {
+  const uint64_t a = v < 0 ? 0 - (uint64_t)v : (uint64_t)v;
+  const int lz = clz64(a);
+  const uint64_t q = lz == 64 ? 0 : a << lz;
+  const uint32_t t = (uint32_t)(q >> 40) | ((q << 24) != 0 ? 1u : 0u);  // 24 bits: exact
+  const uint32_t b = bits_of(i2f(t));
+  const uint32_t r = t == 0 ? 0 : b + ((uint32_t)(40 - kFrac - N - lz) << 23);
+  return f32_of(r | ((uint32_t)((uint64_t)v >> 32) & 0x80000000u));
+}
+
 // ------------------------------------------------------------------ products
 // v = h 2^32 + l with both halves signed, for the product below
 struct Split {
@@ -286,6 +309,52 @@ KBC_HD int clz32(uint32_t x) {
 #endif
 }
 KBC_HD fx shl(fx v, int n) { return (fx)((uint64_t)v << n); }
+
+// f_eq(1 + drho, u) - W for |drho| < 1/4, |u_a| < 1/4: its moments, transformed back; population
+// i times 2^nonzero(i)
+KBC_HD void equilibrium(fx drho, fx ux, fx uy, fx uz, fx (&m)[27]) {
+  const Split ux4 = factor(ux), uy4 = factor(uy), uz4 = factor(uz);
+  const Split third = factor(kThird);
+  const fx ex = axis_e(ux4, ux), ey = axis_e(uy4, uy), ez = axis_e(uz4, uz);
+  const Split wx4 = factor(kThird + mul(split(ex + ex), third));
+  const Split wy4 = factor(kThird + mul(split(ey + ey), third));
+  const Split wz4 = factor(kThird + mul(split(ez + ez), third));
+  const Split rs = split(kOne + drho);
+  const fx rwx = mul(rs, wx4), rwy = mul(rs, wy4);
+  const Split rwxs = split(rwx);
+  m[mi(0, 0, 0)] = drho;
+  m[mi(1, 0, 0)] = mul(rs, ux4);
+  m[mi(0, 1, 0)] = mul(rs, uy4);
+  m[mi(0, 0, 1)] = mul(rs, uz4);
+  const Split jxs = split(m[mi(1, 0, 0)]), jys = split(m[mi(0, 1, 0)]);
+  const Split jzs = split(m[mi(0, 0, 1)]);
+  m[mi(1, 1, 0)] = mul(jxs, uy4);
+  m[mi(1, 0, 1)] = mul(jxs, uz4);
+  m[mi(0, 1, 1)] = mul(jys, uz4);
+  const Split pxys = split(m[mi(1, 1, 0)]);
+  m[mi(1, 2, 0)] = mul(jxs, wy4);
+  m[mi(1, 0, 2)] = mul(jxs, wz4);
+  m[mi(2, 1, 0)] = mul(jys, wx4);
+  m[mi(0, 1, 2)] = mul(jys, wz4);
+  m[mi(2, 0, 1)] = mul(jzs, wx4);
+  m[mi(0, 2, 1)] = mul(jzs, wy4);
+  m[mi(1, 1, 1)] = mul(pxys, uz4);
+  m[mi(2, 1, 1)] = mul(split(m[mi(0, 1, 1)]), wx4);
+  m[mi(1, 2, 1)] = mul(split(m[mi(1, 0, 1)]), wy4);
+  m[mi(1, 1, 2)] = mul(pxys, wz4);
+  m[mi(2, 2, 1)] = mul(split(m[mi(2, 0, 1)]), wy4);
+  m[mi(2, 1, 2)] = mul(split(m[mi(2, 1, 0)]), wz4);
+  m[mi(1, 2, 2)] = mul(split(m[mi(1, 2, 0)]), wz4);
+  m[mi(2, 0, 0)] = rwx - kThird;
+  m[mi(0, 2, 0)] = rwy - kThird;
+  m[mi(0, 0, 2)] = mul(rs, wz4) - kThird;
+  const fx rwxwy = mul(rwxs, wy4);
+  m[mi(2, 2, 0)] = rwxwy - kNinth;
+  m[mi(2, 0, 2)] = mul(rwxs, wz4) - kNinth;
+  m[mi(0, 2, 2)] = mul(split(rwy), wz4) - kNinth;
+  m[mi(2, 2, 2)] = mul(split(rwxwy), wz4) - k27th;
+  to_populations(m);
+}
 
 // the parameters of the collision as integers
 struct Relax {

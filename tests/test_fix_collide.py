@@ -38,6 +38,23 @@ extern "C" void fix_collide(int n, const double* d, double* o, double* g, int* f
     }
   }
 }
+extern "C" void fix_equilibrium(int n, const double* in, double* o, float* of, float* odd) {
+  uint32_t top = 0;
+  for (int k = 0; k < n; ++k) {
+    fix::fx v[4], p[27];
+    for (int a = 0; a < 4; ++a) v[a] = fix::from_f64(in[4 * k + a], &top);
+    fix::equilibrium(v[0], v[1], v[2], v[3], p);
+    for (int i = 0; i < 27; ++i) {
+      const int nz = fix::nonzero(i), j = k * 27 + i;
+      o[j] = nz == 0 ? fix::to_f64<0>(p[i]) : nz == 1 ? fix::to_f64<1>(p[i])
+           : nz == 2 ? fix::to_f64<2>(p[i]) : fix::to_f64<3>(p[i]);
+      of[j] = nz == 0 ? fix::to_f32<0>(p[i]) : nz == 1 ? fix::to_f32<1>(p[i])
+            : nz == 2 ? fix::to_f32<2>(p[i]) : fix::to_f32<3>(p[i]);
+      odd[j] = nz == 0 ? fix::to_f32_odd<0>(p[i]) : nz == 1 ? fix::to_f32_odd<1>(p[i])
+             : nz == 2 ? fix::to_f32_odd<2>(p[i]) : fix::to_f32_odd<3>(p[i]);
+    }
+  }
+}
 extern "C" void fix_round(int n, const double* d, double* o, const float* f, double* of) {
   uint32_t top = 0;
   for (int k = 0; k < n; ++k) {
@@ -199,3 +216,22 @@ def test_conversions(lib):
     unit = 2.0 ** -60
     assert np.array_equal(o, np.trunc(d.astype(LD) / LD(unit)).astype(np.float64) * unit)
     assert np.array_equal(of, np.trunc(f.astype(LD) / LD(unit)).astype(np.float64) * unit)
+
+
+def test_equilibrium_and_its_roundings(lib):
+    """f_eq - W in fixed point, and its roundings to FP32 (to nearest; to odd, after which a
+    rounding to half is the rounding of the exact value)."""
+    rng = np.random.default_rng(4)
+    n = 4000
+    x = np.concatenate([rng.uniform(-0.2, 0.2, (n, 4)), np.zeros((1, 4)),
+                        rng.uniform(-1e-5, 1e-5, (n, 4))])
+    o = np.empty((len(x), 27))
+    of, odd = np.empty((len(x), 27), np.float32), np.empty((len(x), 27), np.float32)
+    lib.fix_equilibrium(len(x), *[a.ctypes.data_as(ctypes.c_void_p) for a in (x, o, of, odd)])
+    ref = product_equilibrium(1 + x[:, 0].astype(LD), x[:, 1:].T.astype(LD), LD) - weights(LD)
+    assert np.abs(o - ref).max() <= 16 * 2.0 ** -57  # |u| up to 0.2: e is good to 2^-54
+    assert np.abs(o - ref)[n + 1:].max() <= 16 * 2.0 ** -60
+    assert not o[n].any() and not of[n].any() and not odd[n].any()
+    # o is exact here for |v| < 2^53 units and rounded above; FP32 of either is the same
+    assert np.array_equal(of, o.astype(np.float32))
+    assert np.array_equal(odd.astype(np.float16), o.astype(np.float16))
