@@ -174,45 +174,26 @@ __device__ __forceinline__ void moments_fp64(const T (&d)[27], double& drho, dou
   m[2] = mz;
 }
 
-// rho and u of canonical f(t). The shifts of a node are scaled to integers by the node's largest
-// exponent (57 bits below it, so the sums are at least as exact as FP64 sums), summed, and the
-// four sums converted; u is rho u times the reciprocal of rho. FP16: the shifts times 216 are
-// exact FP32 numbers (the weights are 64 : 16 : 4 : 1).
-template <typename S, int KIND>
-__global__ void __launch_bounds__(256) moments_kernel(const S* buf, Geo g, double* rho_out,
-                                                      double* u_out, uint64_t n0, uint64_t cnt,
-                                                      uint64_t ld) {
-  using T = typename std::conditional<std::is_same<S, double>::value, double, float>::type;
-  constexpr bool kHalf = std::is_same<S, uint16_t>::value;
+// rho - 1 and u of 27 shifts (FP16: of shifts times 216, see load_shifts), in FP64. The shifts of a
+// node are scaled to integers by the node's largest exponent (57 bits below it, so the sums are
+// at least as exact as FP64 sums), summed, and the four sums converted; u is rho u times the
+// reciprocal of rho. m, if given, receives rho u.
+template <bool HALF, typename T>
+__device__ __forceinline__ void velocity(const T (&d)[27], double& drho, double (&u)[3],
+                                         double* m = nullptr) {
   constexpr int kMant = std::is_same<T, double>::value ? 52 : 23;
   constexpr int kBias = std::is_same<T, double>::value ? 1023 : 127;
-  const uint64_t k = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-  if (k >= cnt) return;
-  uint32_t x, y, z;
-  node_coords(g, n0 + k, x, y, z);
-  Nbr nb;
-  nb.init(g, x, y, z);
-  T d[27];
+  constexpr int kShift = sizeof(T) == 8 ? 20 : 23;
   uint32_t top = 0;  // the largest sign-free high word
-  Unroll<0, 27>::run([&](auto ic) {
-    constexpr int I = decltype(ic)::value;
-    const S v = *canon_ptr<KIND, I>(buf, g, nb);
-    if constexpr (kHalf)
-      d[I] = __fmul_rn(__half2float(__ushort_as_half(v)), (float)(216.0 * wgt(I)));
-    else
-      d[I] = v;
-  });
 #pragma unroll
   for (int i = 0; i < 27; ++i) {
     const uint32_t a = (uint32_t)(fix::bits_of(d[i]) >> (sizeof(T) == 8 ? 32 : 0)) & 0x7fffffffu;
     top = a > top ? a : top;
   }
-  constexpr int kShift = sizeof(T) == 8 ? 20 : 23;
   const int et = (int)(top >> kShift);  // biased exponent of the largest
-  double drho, m[3], ir;
   // the fast path: the largest value between 2^-100 and 1/4 (FP16: 54), rho within the range of
   // the fixed-point reciprocal
-  bool fast = et > kBias - 100 && et < kBias - 2 + (kHalf ? 8 : 0);
+  bool fast = et > kBias - 100 && et < kBias - 2 + (HALF ? 8 : 0);
   if (fast) {
     fix::fx v[27];
 #pragma unroll
@@ -247,30 +228,70 @@ __global__ void __launch_bounds__(256) moments_kernel(const S* buf, Geo g, doubl
       val[j] = __hiloint2double(h == 0 ? 0 : h + ex * (1 << 20), __double2loint(c));
     }
     drho = val[0];
-    if constexpr (kHalf) drho *= 1.0 / 216.0;
+    if constexpr (HALF) drho *= 1.0 / 216.0;
     // rho in units of 2^-60 (FP16: 216 rho in units of 2^-52)
-    const int sh = ex + (kHalf ? 52 : 60);
+    const int sh = ex + (HALF ? 52 : 60);
     const fix::fx ds = sh >= 0 ? fix::shl(sum[0], sh) : (sh < -63 ? 0 : sum[0] >> -sh);
-    const fix::fx r = kHalf ? (216ll << 52) + ds : fix::kOne + ds;
+    const fix::fx r = HALF ? (216ll << 52) + ds : fix::kOne + ds;
     fast = r > fix::kOne / 2 && r < 2 * fix::kOne;
     if (fast) {
       // 1 / rho, or 1 / (216 rho) = 2^-8 / (r 2^-60)
-      ir = fix::to_f64<kHalf ? 8 : 0>(fix::reciprocal(r));
+      const double ir = fix::to_f64<HALF ? 8 : 0>(fix::reciprocal(r));
 #pragma unroll
-      for (int a = 0; a < 3; ++a) m[a] = __dmul_rn(val[a + 1], ir);
+      for (int a = 0; a < 3; ++a) {
+        u[a] = __dmul_rn(val[a + 1], ir);
+        if (m) m[a] = HALF ? val[a + 1] * (1.0 / 216.0) : val[a + 1];
+      }
     }
   }
   if (!fast) {
-    moments_fp64(d, drho, m);
-    if constexpr (kHalf) {
-      drho /= 216.0;
-      for (int a = 0; a < 3; ++a) m[a] /= 216.0;
+    double j[3];
+    moments_fp64(d, drho, j);
+    if constexpr (HALF) drho /= 216.0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      if constexpr (HALF) j[a] /= 216.0;
+      if (m) m[a] = j[a];
+      u[a] = j[a] / (1.0 + drho);
     }
-    for (int a = 0; a < 3; ++a) m[a] /= 1.0 + drho;
   }
+}
+
+// The shifts of a node for velocity(). FP16: times 216, which are exact FP32 numbers (the weights
+// are 64 : 16 : 4 : 1).
+template <typename S> struct ShiftType { using T = float; };
+template <> struct ShiftType<double> { using T = double; };
+template <typename S, int KIND>
+__device__ __forceinline__ void load_shifts(const S* buf, const Geo& g, const Nbr& nb,
+                                            typename ShiftType<S>::T (&d)[27]) {
+  Unroll<0, 27>::run([&](auto ic) {
+    constexpr int I = decltype(ic)::value;
+    const S v = *canon_ptr<KIND, I>(buf, g, nb);
+    if constexpr (std::is_same<S, uint16_t>::value)
+      d[I] = __fmul_rn(__half2float(__ushort_as_half(v)), (float)(216.0 * wgt(I)));
+    else
+      d[I] = v;
+  });
+}
+
+// rho and u of canonical f(t)
+template <typename S, int KIND>
+__global__ void __launch_bounds__(256) moments_kernel(const S* buf, Geo g, double* rho_out,
+                                                      double* u_out, uint64_t n0, uint64_t cnt,
+                                                      uint64_t ld) {
+  const uint64_t k = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+  if (k >= cnt) return;
+  uint32_t x, y, z;
+  node_coords(g, n0 + k, x, y, z);
+  Nbr nb;
+  nb.init(g, x, y, z);
+  typename ShiftType<S>::T d[27];
+  load_shifts<S, KIND>(buf, g, nb, d);
+  double drho, u[3];
+  velocity<std::is_same<S, uint16_t>::value>(d, drho, u);
   if (rho_out) rho_out[k] = 1.0 + drho;
 #pragma unroll
-  for (int a = 0; a < 3; ++a) u_out[a * ld + k] = m[a];
+  for (int a = 0; a < 3; ++a) u_out[a * ld + k] = u[a];
 }
 
 // f_eq(rho, u) in FP64 instructions, stored (FP64 storage, and nodes off the fixed-point range)
@@ -327,21 +348,45 @@ __global__ void __launch_bounds__(256) init_kernel(S* buf, Geo g, const double* 
 // ------------------------------------------------------------------ diagnostics
 // Sums (FP64) in partials[block * kDiagSums + j], over the nodes whose rho and u are finite
 // (0-10) or whose velocity gradients are finite (11-19):
-//  0 sum (rho - 1), 1-3 sum rho u, 4-6 sum u, 7 sum |u|^2, 8 sum gamma, 9 sum gamma^2,
+//  0 sum (rho - 1), 1-3 sum rho u, 4-6 sum u, 7 unused, 8 sum gamma, 9 sum gamma^2,
 //  10 non-finite nodes, 11 sum |curl u|^2, 12 sum (d_b u_a + d_a u_b)^2,
 //  13-17 sum (d u_x / d x)^n for n = 2..6, 18 sum |u - <u>|^2 (second pass, with <u> from the
 //  first), 19 nodes with finite gradients
-template <int N>
-__device__ __forceinline__ void block_reduce_store(double (&v)[N], double* dst) {
-  __shared__ double sh[32][N];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+//
+// Warp sums by halving: a lane gives half of its values away at each step and adds the other
+// half's, so that N <= 16 values cost 16 FP64 additions a lane and not 5 N (on GB300's FP64 pipe
+// the trees of 11 and 9 values took most of a 32^3 diagnostics' 40 us).
+template <int O, int M>
+__device__ __forceinline__ void halve(double (&v)[M > 0 ? 2 * M : 1], int lane, int& slot,
+                                      double& sum) {
+  if constexpr (M == 0) {
+    sum = v[0];
 #pragma unroll
-  for (int j = 0; j < N; ++j) {
+    for (int o = O; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  } else {
+    const bool up = lane & O;
+    double w[M];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[j] += __shfl_down_sync(0xffffffffu, v[j], o);
+    for (int j = 0; j < M; ++j) {
+      const double give = up ? v[j] : v[j + M], keep = up ? v[j + M] : v[j];
+      w[j] = keep + __shfl_xor_sync(0xffffffffu, give, O);
+    }
+    if (up) slot += M;
+    halve<O / 2, M / 2>(w, lane, slot, sum);
   }
-  if (lane == 0)
-    for (int j = 0; j < N; ++j) sh[warp][j] = v[j];
+}
+
+template <int N>
+__device__ __forceinline__ void block_reduce_store(const double (&in)[N], double* dst) {
+  constexpr int M = N > 8 ? 16 : 8;
+  __shared__ double sh[32][M];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double v[M], sum;
+#pragma unroll
+  for (int j = 0; j < M; ++j) v[j] = j < N ? in[j] : 0.0;
+  int slot = 0;
+  halve<16, M / 2>(v, lane, slot, sum);
+  if ((lane & (32 / M - 1)) == 0) sh[warp][slot] = sum;
   __syncthreads();
   if (threadIdx.x < N) {
     double acc = 0.0;
@@ -349,6 +394,14 @@ __device__ __forceinline__ void block_reduce_store(double (&v)[N], double* dst) 
     for (int w = 0; w < nw; ++w) acc += sh[w][threadIdx.x];
     dst[threadIdx.x] = acc;
   }
+}
+
+// isfinite() without the FP64 pipe's compare
+__device__ __forceinline__ bool finite_bits(double v) {
+  return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000;
+}
+__device__ __forceinline__ bool finite_bits(float v) {
+  return (__float_as_uint(v) & 0x7f800000u) != 0x7f800000u;
 }
 
 // rho - 1 and rho u of canonical f(t) at one node, in the arithmetic type of the storage
@@ -373,9 +426,10 @@ __device__ __forceinline__ void node_moments_r(const S* buf, const Geo& g, const
 }
 
 // Per-node quantities in the storage's arithmetic type; block and global sums in FP64.
-// 4 blocks of 256 threads per SM: the fixed grid of 608 blocks is then resident in one wave
+// 4 blocks of 256 threads per SM: the fixed grid of 608 blocks is then resident in one wave (FP64:
+// 2 blocks, whose integer sums need 128 registers)
 template <typename S, int KIND>
-__global__ void __launch_bounds__(256, 4) diag_fields_kernel(const S* buf, Geo g,
+__global__ void __launch_bounds__(256, std::is_same<S, double>::value ? 2 : 4) diag_fields_kernel(const S* buf, Geo g,
                                                           const float* gamma, int with_gamma,
                                                           typename Codec<S>::R* uf,
                                                           double* partials) {
@@ -389,15 +443,23 @@ __global__ void __launch_bounds__(256, 4) diag_fields_kernel(const S* buf, Geo g
     node_coords(g, n, x, y, z);
     Nbr nb;
     nb.init(g, x, y, z);
-    R drho, m[3];
-    node_moments_r<S, KIND>(buf, g, nb, drho, m);
+    R drho, m[3], ux, uy, uz;
+    if constexpr (std::is_same<S, double>::value) {
+      // integer sums: the FP64 pipe would take 130 operations a node for the moments
+      double d[27], uu[3];
+      load_shifts<S, KIND>(buf, g, nb, d);
+      velocity<false>(d, drho, uu, m);
+      ux = uu[0], uy = uu[1], uz = uu[2];
+    } else {
+      node_moments_r<S, KIND>(buf, g, nb, drho, m);
+      const R ir = R(1) / (R(1) + drho);
+      ux = m[0] * ir, uy = m[1] * ir, uz = m[2] * ir;
+    }
     const R rho = R(1) + drho;
-    const R ir = R(1) / rho;
-    const R ux = m[0] * ir, uy = m[1] * ir, uz = m[2] * ir;
     uf[n] = ux;
     uf[g.P + n] = uy;
     uf[2 * g.P + n] = uz;
-    if (!isfinite(rho) || !isfinite(ux) || !isfinite(uy) || !isfinite(uz)) {
+    if (!finite_bits(rho) || !finite_bits(ux) || !finite_bits(uy) || !finite_bits(uz)) {
       acc[10] += R(1);
       continue;
     }
@@ -408,7 +470,6 @@ __global__ void __launch_bounds__(256, 4) diag_fields_kernel(const S* buf, Geo g
     acc[4] += ux;
     acc[5] += uy;
     acc[6] += uz;
-    acc[7] += ux * ux + uy * uy + uz * uz;
     if (with_gamma) {
       const R gm = (R)gamma[n];
       acc[8] += gm;
@@ -483,7 +544,7 @@ __global__ void __launch_bounds__(256) diag_grad_kernel(Geo g, const R* uf, cons
         const R s = gr[a][b] + gr[b][a];
         ss += s * s;
       }
-    if (isfinite(ww) && isfinite(ss)) {
+    if (finite_bits(ww) && finite_bits(ss)) {
       acc[0] += ww;
       acc[1] += ss;
       const R q = gr[0][0];
@@ -497,7 +558,7 @@ __global__ void __launch_bounds__(256) diag_grad_kernel(Geo g, const R* uf, cons
     }
     const R d0 = uf[n] - mean[0], d1 = uf[g.P + n] - mean[1], d2 = uf[2 * g.P + n] - mean[2];
     const R dd = d0 * d0 + d1 * d1 + d2 * d2;
-    if (isfinite(dd)) acc[7] += dd;
+    if (finite_bits(dd)) acc[7] += dd;
   }
   double v[9];
 #pragma unroll
@@ -505,13 +566,23 @@ __global__ void __launch_bounds__(256) diag_grad_kernel(Geo g, const R* uf, cons
   block_reduce_store<9>(v, partials + blockIdx.x * kDiagSums + 11);
 }
 
-// fixed-order final reduction: sums[j] = sum over blocks of partials[block][j]
-static __global__ void diag_final_kernel(const double* partials, int nblocks, double* sums) {
-  const int j = threadIdx.x;
-  if (j >= kDiagSums) return;
+// Fixed-order final reduction of the slots [first, first + blockDim.x / 32): sums[j] = sum over
+// blocks of partials[block][j], a warp per slot (each lane every 32nd block, then the lanes). One
+// thread per slot over 608 blocks took 54 us a call, as long as a 32^3 diagnostics otherwise.
+// With counters given, slots 20 and 21 take the guard count and the timeout flag, so that one
+// copy brings the host everything.
+static __global__ void diag_final_kernel(const double* partials, int nblocks, int first,
+                                         double* sums, const StepCounters* ctr) {
+  const int j = first + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   double acc = 0.0;
-  for (int b = 0; b < nblocks; ++b) acc += partials[b * kDiagSums + j];
-  sums[j] = acc;
+  for (int b = lane; b < nblocks; b += 32) acc += partials[b * kDiagSums + j];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+  if (lane == 0) sums[j] = acc;
+  if (ctr && threadIdx.x == 0) {
+    sums[20] = (double)ctr->guarded;
+    sums[21] = (double)ctr->timeout;
+  }
 }
 
 // Stabilizer gap on canonical f(t): per node the estimate eq:result21 and the root of
@@ -567,16 +638,20 @@ __global__ void __launch_bounds__(256) gap_kernel(const S* b0, const S* b1, Geo 
   }
 }
 
-// fixed-order final reduction of the gap partials (slot 6 by maximum)
+// fixed-order final reduction of the gap partials, a warp per slot (slot 6 by maximum)
 static __global__ void gap_final_kernel(const double* partials, int nblocks, double* sums) {
-  const int j = threadIdx.x;
-  if (j >= kGapSums) return;
+  const int j = threadIdx.x >> 5, lane = threadIdx.x & 31;
   double acc = 0.0;
-  for (int b = 0; b < nblocks; ++b) {
+  for (int b = lane; b < nblocks; b += 32) {
     const double p = partials[b * kDiagSums + j];
     acc = j == 6 ? fmax(acc, p) : acc + p;
   }
-  sums[j] = acc;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double p = __shfl_down_sync(0xffffffffu, acc, o);
+    acc = j == 6 ? fmax(acc, p) : acc + p;
+  }
+  if (lane == 0) sums[j] = acc;
 }
 
 // ------------------------------------------------------------------ density pre-solve
@@ -763,16 +838,18 @@ cudaError_t Ops<S>::gamma_gap(const BoxView& b, int64_t t, double* partials, int
   else
     gap_kernel<S, false><<<nblocks, 256, 0, st>>>((const S*)b.pop[0], (const S*)b.pop[1], g,
                                                   b.scheme, (int)(t & 1), cp, partials);
-  gap_final_kernel<<<1, 32, 0, st>>>(partials, nblocks, sums);
+  gap_final_kernel<<<1, 32 * kGapSums, 0, st>>>(partials, nblocks, sums);
   return cudaGetLastError();
 }
 
 template <typename S>
 cudaError_t Ops<S>::diag(const BoxView& b, int64_t t, bool with_gamma, int order, void* ufield,
-                         double* partials, int nblocks, double* sums, cudaStream_t st) {
+                         double* partials, int nblocks, double* sums, const StepCounters* ctr,
+                         cudaStream_t st) {
   using R = typename Codec<S>::R;
   const Geo g = make_geo(b);
-  cudaMemsetAsync(partials, 0, sizeof(double) * kDiagSums * nblocks, st);
+  // blocks without a node would only reduce zeros
+  if ((uint64_t)nblocks * 256 > g.P) nblocks = (int)((g.P + 255) / 256);
   const int parity = (int)(t & 1);
   const int wg = with_gamma ? 1 : 0;
   if (b.scheme == 0)
@@ -784,12 +861,14 @@ cudaError_t Ops<S>::diag(const BoxView& b, int64_t t, bool with_gamma, int order
   else
     diag_fields_kernel<S, 2><<<nblocks, 256, 0, st>>>((const S*)b.pop[0], g, b.gamma, wg,
                                                       (R*)ufield, partials);
-  diag_final_kernel<<<1, 32, 0, st>>>(partials, nblocks, sums);  // <u> for the second pass
+  if (order == 0) return cudaGetLastError();
+  // <u> for the second pass
+  diag_final_kernel<<<1, 11 * 32, 0, st>>>(partials, nblocks, 0, sums, nullptr);
   if (order == 8)
     diag_grad_kernel<R, 4><<<nblocks, 256, 0, st>>>(g, (const R*)ufield, sums, partials);
   else
     diag_grad_kernel<R, 1><<<nblocks, 256, 0, st>>>(g, (const R*)ufield, sums, partials);
-  diag_final_kernel<<<1, 32, 0, st>>>(partials, nblocks, sums);
+  diag_final_kernel<<<1, 9 * 32, 0, st>>>(partials, nblocks, 11, sums, ctr);
   return cudaGetLastError();
 }
 

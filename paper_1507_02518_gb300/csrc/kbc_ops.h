@@ -97,9 +97,11 @@ template <typename S> struct Ops {
   static cudaError_t moments(const BoxView& b, int64_t t, double* rho, double* u, uint64_t n0,
                              uint64_t cnt, uint64_t ld, cudaStream_t st);
   // diagnostics: writes u (arithmetic type of S) to ufield[3][P] and per-block partial sums
-  // order: 2 or 8, the order of the central differences of the velocity gradients
+  // order: 2 or 8, the order of the central differences of the velocity gradients (0: the
+  // velocity field only); sums[20], sums[21] take the guard count and timeout flag of ctr
   static cudaError_t diag(const BoxView& b, int64_t t, bool with_gamma, int order, void* ufield,
-                          double* partials, int nblocks, double* sums, cudaStream_t st);
+                          double* partials, int nblocks, double* sums, const StepCounters* ctr,
+                          cudaStream_t st);
   // one density pre-solve iteration t -> t+1 with the velocity held at u0 ([3][P], collision
   // precision); `store` keeps rho - 1 of f(t) in b.gamma for rho_change
   static cudaError_t presolve_step(const BoxView& b, int64_t t, double beta_pre, const void* u0,
