@@ -28,9 +28,15 @@ template <> struct MaxThreads<double> { static constexpr int value = 256; };
 // ends. What it hides is the launch latency between kernels and the start of the next one behind
 // the last blocks of this: 32^3 FP32 AA (step and pass) 9.2 -> 5.4 us a step with the node order
 // below, 256^3 pull 542 -> 537 us. Launched without the attribute, follow() does nothing.
+// Where waiting blocks take places that unbalance the next kernel over the SMs, the next one is
+// let in at the end only: the pull step (let_next(): 32^3 3.9 -> 3.4 us, 48^3 5.2 -> 4.9; the AA
+// step is better with follow(), 4.4 against 4.7), and the FP64 step, whose blocks fill an SM with
+// three, when they exit (32^3 11.2 -> 8.7 us).
+__device__ __forceinline__ void wait_before() { cudaGridDependencySynchronize(); }
+__device__ __forceinline__ void let_next() { cudaTriggerProgrammaticLaunchCompletion(); }
 __device__ __forceinline__ void follow() {
-  cudaTriggerProgrammaticLaunchCompletion();
-  cudaGridDependencySynchronize();
+  let_next();
+  wait_before();
 }
 template <typename... P, typename... A>
 static cudaError_t launch_following(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st,
@@ -67,7 +73,7 @@ template <int MODE, bool RECORD>
 __global__ void __maxnreg__(168) fix_step_kernel(const double* src, double* dst, Geo g,
                                                          CollideParams cp, float* gamma_out,
                                                          StepCounters* ctr) {
-  follow();
+  wait_before();
   const uint32_t n = g.zb * g.nxy + blockIdx.x * blockDim.x + threadIdx.x;  // P < 2^31
   if (n >= g.ze * g.nxy) return;
   const uint32_t row = n / g.nx;
@@ -116,11 +122,13 @@ template <typename S, int MODE, bool RECORD>
 __global__ void __launch_bounds__(128, 3) adj_step_kernel(const S* src, S* dst, Geo g,
                                                        CollideParams cp, float* gamma_out,
                                                        StepCounters* ctr) {
-  follow();
+  if (MODE != MODE_PULL) let_next();
+  wait_before();
   const uint32_t x = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
   if (x >= g.nx) return;
   node_update_adj<S, MODE, RECORD>(src, dst, g, x, blockIdx.y, blockIdx.z + g.zb, cp,
                                    gamma_out, ctr);
+  if (MODE == MODE_PULL) let_next();
 }
 
 // The same over the box's node order: pair k is nodes (2k, 2k + 1), which share a row as nx is
@@ -131,13 +139,15 @@ template <typename S, int MODE, bool RECORD>
 __global__ void __launch_bounds__(128, 3) adj_linear_kernel(const S* src, S* dst, Geo g,
                                                          CollideParams cp, float* gamma_out,
                                                          StepCounters* ctr) {
-  follow();
+  if (MODE != MODE_PULL) let_next();
+  wait_before();
   const uint32_t n = g.zb * g.nxy + 2 * (blockIdx.x * blockDim.x + threadIdx.x);  // P < 2^31
   if (n >= g.ze * g.nxy) return;
   const uint32_t row = n / g.nx;
   const uint32_t z = row / g.ny;
   node_update_adj<S, MODE, RECORD>(src, dst, g, n - row * g.nx, row - z * g.ny, z, cp, gamma_out,
                                    ctr);
+  if (MODE == MODE_PULL) let_next();
 }
 
 // Rows of a multiple of 64 nodes: blocks of whole row segments; other rows: the node order.
