@@ -880,8 +880,8 @@ __device__ __forceinline__ R collide(R (&d)[27], const CollideParams& cp, int* g
 //     velocities -1, 0, +1 as 1 : 4 : 1 (that is 6 W_v), so the moments come out 216 times
 //     their value; that factor and the 1/W_i of the outputs sit in the constants of Table 1's
 //     class values, and dh/W = h - G - ds/W needs no weight per population;
-//   * the entropic weights (W_i/f_eq_i for REL, 1/f_eq_i otherwise) are products of one MUFU
-//     reciprocal per axis and velocity component;
+//   * the entropic weights 1/f_eq_i are products of one MUFU reciprocal per axis and velocity
+//     component, for REL (W_i/f_eq_i up to a common factor) of factors without a reciprocal;
 //   * the q part's switch multiplies three class constants, not the seven third moments;
 //   * 3u^2 reuses 3u, and the first term of each entropic sum is a product, not an FMA on 0.
 template <typename R, bool REL>
@@ -1031,15 +1031,30 @@ __device__ __forceinline__ R collide_lean(R (&d)[27], const CollideParams& cp, i
   fz[0] = O::sub(tez, uz3);
   fz[1] = O::neg(ez);
   fz[2] = O::add(tez, uz3);
-  // entropic weights per axis: REL W_a / X_a, otherwise 1 / (W_a X_a)
+  // entropic weights per axis: 1 / (W_a X_a), for REL W_a / X_a
   R wx[3], wy[3], wz[3];
+  if constexpr (REL) {
+    // up to factors common to an axis, which drop out of gamma's ratio, 1 / X_+- is X_-+ and 1 / X_0 is
+    // X_0 (the product form has X_+ X_- = X_0^2; rho is such a factor too): no reciprocals
+    const R c6 = O::c(1.0 / 6.0);
+    auto axis_w = [&](R te, R u3, R e, R (&w)[3]) {
+      const R b = O::fma(te, c6, c6), u6 = O::mul(u3, c6);
+      w[0] = O::add(b, u6);
+      w[1] = O::fma(O::neg(c23), e, c23);
+      w[2] = O::sub(b, u6);
+    };
+    axis_w(tex, ux3, ex, wx);
+    axis_w(tey, uy3, ey, wy);
+    axis_w(tez, uz3, ez, wz);
+  } else {
+    // (<dh|dh> itself is compared with kDenFp64 here)
 #pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    const double Wa = a == 1 ? 2.0 / 3.0 : 1.0 / 6.0;
-    const R cw = O::c(REL ? 1.0 / Wa : Wa);
-    wx[a] = O::rcp_fast(O::fma(cw, gx[a], cw));
-    wy[a] = O::rcp_fast(O::fma(cw, fy[a], cw));
-    wz[a] = O::rcp_fast(O::fma(cw, fz[a], cw));
+    for (int a = 0; a < 3; ++a) {
+      const R cw = O::c(a == 1 ? 2.0 / 3.0 : 1.0 / 6.0);
+      wx[a] = O::rcp_fast(O::fma(cw, gx[a], cw));
+      wy[a] = O::rcp_fast(O::fma(cw, fy[a], cw));
+      wz[a] = O::rcp_fast(O::fma(cw, fz[a], cw));
+    }
   }
   // X_a Y_b - 1 for the 9 (a, b) pairs, without cancellation
   R Pab[9];
@@ -1507,13 +1522,29 @@ __device__ __forceinline__ void node_update_adj(const S* src, S* dst, const Geo&
   oz[2] = (z + 1 == g.nz ? 0 : z + 1) * g.nxy;
   uint32_t xm = x == 0 ? g.nx - 1 : x - 1;
   uint32_t xp2 = x + 2 == g.nx ? 0 : x + 2;
+  // The address of node xx of a row: FP16 by a 32-bit byte offset (2 P < 2^32) from the plane's
+  // address, which is the same for all threads, so that no access needs a 64-bit multiply-add of
+  // its own (256^3 AA with the prefetch: 381 -> 376 us); FP32 from the row's address (offsets of
+  // both kinds live across the collision spilled).
+  auto at = [](auto* plane, uint32_t o1, uint32_t o2, uint32_t xx) {
+    if constexpr (std::is_same<S, uint16_t>::value) {
+      using Q = decltype(plane);
+      using B = typename std::conditional<
+          std::is_const<typename std::remove_pointer<Q>::type>::value, const char, char>::type;
+      return reinterpret_cast<Q>(reinterpret_cast<B*>(plane) + (uint32_t)(2u * (o1 + o2 + xx)));
+    } else {
+      auto* row = plane + o1 + o2;
+      return row + xx;
+    }
+  };
   float2 d[27];
   Unroll<0, 27>::run([&](auto ic) {
     constexpr int I = decltype(ic)::value;
     constexpr int LS = Pat::load_shift;
-    const S* row = src + (uint64_t)Pat::load_plane(I) * g.P + oy[LS * cy(I) + 1] +
-                   oz[LS * cz(I) + 1];
-    d[I] = IO::template get<LS * cx(I), MODE == MODE_PULL>(row + x, row + xm, row + xp2);
+    const S* plane = src + (uint64_t)Pat::load_plane(I) * g.P;
+    const uint32_t o1 = oy[LS * cy(I) + 1], o2 = oz[LS * cz(I) + 1];
+    d[I] = IO::template get<LS * cx(I), MODE == MODE_PULL>(
+        at(plane, o1, o2, x), at(plane, o1, o2, xm), at(plane, o1, o2, xp2));
   });
   int guarded, fp64 = 0;
   float2 gamma = collide_step<float2, false, false, false, C::rel>(
@@ -1544,21 +1575,22 @@ __device__ __forceinline__ void node_update_adj(const S* src, S* dst, const Geo&
   Unroll<0, 27>::run([&](auto ic) {
     constexpr int I = decltype(ic)::value;
     constexpr int SS = Pat::store_shift;
-    S* row = dsts + (uint64_t)Pat::store_plane(I) * Ps + oy[SS * cy(I) + 1] + oz[SS * cz(I) + 1];
+    S* plane = dsts + (uint64_t)Pat::store_plane(I) * Ps;
+    const uint32_t o1 = oy[SS * cy(I) + 1], o2 = oz[SS * cz(I) + 1];
     constexpr int SX = SS * cx(I);
     if constexpr (SX == 0) {
       if (!skip) {
-        IO::put2(row + x, d[I]);
+        IO::put2(at(plane, o1, o2, x), d[I]);
       } else {
-        if (wa) IO::put1(row + x, d[I].x);
-        if (wb) IO::put1(row + x + 1, d[I].y);
+        if (wa) IO::put1(at(plane, o1, o2, x), d[I].x);
+        if (wb) IO::put1(at(plane, o1, o2, x + 1), d[I].y);
       }
     } else if constexpr (SX > 0) {
-      if (wa) IO::put1(row + x + 1, d[I].x);
-      if (wb) IO::put1(row + xp2, d[I].y);
+      if (wa) IO::put1(at(plane, o1, o2, x) + 1, d[I].x);
+      if (wb) IO::put1(at(plane, o1, o2, xp2), d[I].y);
     } else {
-      if (wa) IO::put1(row + xm, d[I].x);
-      if (wb) IO::put1(row + x, d[I].y);
+      if (wa) IO::put1(at(plane, o1, o2, xm), d[I].x);
+      if (wb) IO::put1(at(plane, o1, o2, x), d[I].y);
     }
   });
   if (fp64) {

@@ -99,6 +99,32 @@ __device__ __forceinline__ void advance_node(uint32_t& x, uint32_t& y, uint32_t&
   }
 }
 
+// Brings into L2 what the blocks one wave ahead will load (kWave blocks are resident on the
+// chip: 3 on each of 152 SMs): the warp's share of the 27 planes of the tile that starts kWave
+// blocks after node n, a 128-byte line per lane. With 12 warps per SM the loads' latency is what
+// the step waits for. us a step without -> with: adjacent pairs FP16 256^3 AA 411 -> 378, pull 383
+// -> 367, 200^3 AA 229 -> 193, FP32 AA 256^3 551 -> 534, 200^3 (node order) 321 -> 264; pairs
+// (n, n + 32) FP32 201^3 AA 321 -> 293, pull 292 -> 287, FP16 269 -> 241, 243 -> 218, central moments
+// FP32 192^3 pull 268 -> 257. The adjacent-pair FP32 pull step, at the DRAM rate already, lost
+// (537 -> 560) and does without. (200 or 912 blocks ahead: FP16 AA 391, 390. Loading the next tile
+// into registers instead takes 238 of them, 8 warps per SM: 438.)
+constexpr uint32_t kWave = 456;
+template <typename S>
+__device__ __forceinline__ void prefetch_ahead(const S* src, const Geo& g, uint64_t n) {
+  const uint32_t lane = threadIdx.x & 31;
+  n += (uint64_t)kWave * 2 * blockDim.x + 2 * (threadIdx.x & ~31u);
+  if (lane < 27 && n < g.P) {
+    const S* p = src + (uint64_t)lane * g.P + n;
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+    // FP32: the second half of the warp's 64 nodes
+    if (sizeof(S) == 4 && n + 32 < g.P) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + 32));
+  }
+}
+// where it is worth its instructions: populations larger than L2 (129 MB)
+template <typename S> __host__ __device__ inline bool beyond_l2(const Geo& g) {
+  return 27 * g.P * sizeof(S) > (129ull << 20);
+}
+
 // Two nodes per thread with packed FP32x2 arithmetic: a block of up to 128 threads covers
 // 2 x blockDim.x consecutive x nodes of one row, each warp 64 of them as (x, x + 32) pairs.
 template <typename S, int MODE, bool RECORD, bool CENTRAL, bool POLY = false>
@@ -109,6 +135,9 @@ __global__ void __launch_bounds__(128, 3) pair_step_kernel(const S* src, S* dst,
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t xa = blockIdx.x * (2 * blockDim.x) + warp * 64 + lane;
   if (xa >= g.nx) return;
+  if (beyond_l2<S>(g))
+    prefetch_ahead<S>(src, g, (uint64_t)(blockIdx.z + g.zb) * g.nxy +
+                                  (uint64_t)blockIdx.y * g.nx + blockIdx.x * (2 * blockDim.x));
   const bool vb = xa + 32 < g.nx;
   const uint32_t z = blockIdx.z + g.zb;
   node_update2<S, MODE, RECORD, CENTRAL, POLY>(src, dst, g, xa, blockIdx.y, z,
@@ -118,12 +147,15 @@ __global__ void __launch_bounds__(128, 3) pair_step_kernel(const S* src, S* dst,
 
 // Two adjacent nodes per thread, (x, x + 1) with x even: a block of blockDim.x threads covers
 // 2 blockDim.x consecutive nodes of one row (nx even).
-template <typename S, int MODE, bool RECORD>
+template <typename S, int MODE, bool RECORD, bool AHEAD>
 __global__ void __launch_bounds__(128, 3) adj_step_kernel(const S* src, S* dst, Geo g,
                                                        CollideParams cp, float* gamma_out,
                                                        StepCounters* ctr) {
   if (MODE != MODE_PULL) let_next();
   wait_before();
+  if constexpr (AHEAD)
+    prefetch_ahead<S>(src, g, (uint64_t)(blockIdx.z + g.zb) * g.nxy +
+                                  (uint64_t)blockIdx.y * g.nx + 2 * blockIdx.x * blockDim.x);
   const uint32_t x = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
   if (x >= g.nx) return;
   node_update_adj<S, MODE, RECORD>(src, dst, g, x, blockIdx.y, blockIdx.z + g.zb, cp,
@@ -135,7 +167,7 @@ __global__ void __launch_bounds__(128, 3) adj_step_kernel(const S* src, S* dst, 
 // even. For rows that are no multiple of 64 nodes this keeps every lane busy (at 32 nodes half of a
 // warp idled), at the price of two divisions per thread: FP32 pull 48^3 11.3 -> 5.2 us, 200^3 303 ->
 // 268, FP32 AA 96^3 41 -> 34 (with the overlapped launches).
-template <typename S, int MODE, bool RECORD>
+template <typename S, int MODE, bool RECORD, bool AHEAD>
 __global__ void __launch_bounds__(128, 3) adj_linear_kernel(const S* src, S* dst, Geo g,
                                                          CollideParams cp, float* gamma_out,
                                                          StepCounters* ctr) {
@@ -143,6 +175,7 @@ __global__ void __launch_bounds__(128, 3) adj_linear_kernel(const S* src, S* dst
   wait_before();
   const uint32_t n = g.zb * g.nxy + 2 * (blockIdx.x * blockDim.x + threadIdx.x);  // P < 2^31
   if (n >= g.ze * g.nxy) return;
+  if constexpr (AHEAD) prefetch_ahead<S>(src, g, n - 2 * threadIdx.x);
   const uint32_t row = n / g.nx;
   const uint32_t z = row / g.ny;
   node_update_adj<S, MODE, RECORD>(src, dst, g, n - row * g.nx, row - z * g.ny, z, cp, gamma_out,
@@ -155,15 +188,22 @@ template <typename S, int MODE, bool RECORD>
 static cudaError_t launch_adj(const S* src, S* dst, const Geo& g, const CollideParams& cp,
                               float* gamma_out, StepCounters* ctr, cudaStream_t st) {
   const uint32_t pairs = g.nx / 2;
-  if (pairs % 32 != 0) {
-    const uint32_t all = pairs * g.ny * (g.ze - g.zb);
-    return launch_following(adj_linear_kernel<S, MODE, RECORD>, (all + 127) / 128, 128, st, src,
-                            dst, g, cp, gamma_out, ctr);
+  auto run = [&](auto ahead) {
+    constexpr bool A = decltype(ahead)::value;
+    if (pairs % 32 != 0) {
+      const uint32_t all = pairs * g.ny * (g.ze - g.zb);
+      return launch_following(adj_linear_kernel<S, MODE, RECORD, A>, (all + 127) / 128, 128, st,
+                              src, dst, g, cp, gamma_out, ctr);
+    }
+    const uint32_t threads = pairs >= 128 ? 128 : pairs;
+    const dim3 grid((pairs + threads - 1) / threads, g.ny, g.ze - g.zb);
+    return launch_following(adj_step_kernel<S, MODE, RECORD, A>, grid, threads, st, src, dst, g, cp,
+                            gamma_out, ctr);
+  };
+  if constexpr (sizeof(S) == 2 || MODE != MODE_PULL) {
+    if (beyond_l2<S>(g)) return run(std::true_type{});
   }
-  const uint32_t threads = pairs >= 128 ? 128 : pairs;
-  const dim3 grid((pairs + threads - 1) / threads, g.ny, g.ze - g.zb);
-  return launch_following(adj_step_kernel<S, MODE, RECORD>, grid, threads, st, src, dst, g, cp,
-                          gamma_out, ctr);
+  return run(std::false_type{});
 }
 
 // The same update over the box's node order instead of rows: block k covers nodes
@@ -179,6 +219,7 @@ __global__ void __launch_bounds__(128, 3) pair_linear_kernel(const S* src, S* ds
   const uint32_t nend = g.ze * g.nxy;  // P < 2^31
   const uint32_t n = g.zb * g.nxy + blockIdx.x * 256 + warp * 64 + lane;
   if (n >= nend) return;
+  if (beyond_l2<S>(g)) prefetch_ahead<S>(src, g, g.zb * g.nxy + blockIdx.x * 256);
   const uint32_t row = n / g.nx;
   const uint32_t xa = n - row * g.nx;
   const uint32_t za = row / g.ny;

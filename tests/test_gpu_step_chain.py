@@ -77,3 +77,30 @@ def test_steps_in_a_captured_graph():
         g.replay()
     torch.cuda.synchronize()
     assert np.array_equal(lat.get_populations(), want.get_populations())
+
+
+@pytest.mark.parametrize("nx,variant", [(128, "d+t+q"), (130, "d+t+q"), (131, "d+t+q"), (256, "cd+ct+cq")])
+@pytest.mark.parametrize("storage", ["f32", "f16"])
+@pytest.mark.parametrize("scheme", ["pull", "aa"])
+def test_boxes_larger_than_l2(nx, variant, storage, scheme):
+    """Populations over 129 MB take the kernels that prefetch a wave ahead; the same bits as the
+    one-node kernel's (central moments, which have no such kernel here: as steps apart)."""
+    ny, nz = 101, {"f32": 100, "f16": 200}[storage]
+    P = nx * ny * nz
+    assert 27 * P * {"f32": 4, "f16": 2}[storage] > 129 << 20
+    u = 0.04 * torch.randn(3, nz, ny, nx, generator=torch.Generator("cuda").manual_seed(1),
+                           dtype=torch.float64, device="cuda").clamp(-3, 3)
+    out = []
+    for kernel in ("auto", "direct"):
+        lat = lb.Lattice(nx, ny, nz, nu=1e-3, storage=storage, scheme=scheme, variant=variant)
+        if variant == "d+t+q":
+            lat.set_kernel(kernel)
+        lat.init_field(None, u)
+        for n in ((3,) if kernel == "auto" else (1, 1, 1)):
+            lat.step(n)
+            torch.cuda.synchronize()
+        f = torch.empty((27, nz, ny, nx), dtype=torch.float64, device="cuda")
+        lb.lb_get_populations(lat.ctx, f.data_ptr(), True)
+        out.append(f)
+        del lat
+    assert torch.equal(out[0], out[1])
