@@ -1505,10 +1505,12 @@ __device__ __forceinline__ void node_update2(const S* src, S* dst, const Geo& g,
 // even AA step, written as one 32/64-bit access per plane; the x-shifted ones as two scalar
 // accesses. The 9 neighbour rows are addressed from 3 + 3 row offsets and 3 x positions,
 // which keeps fewer registers live than two full neighbourhoods. FP32 arithmetic only.
-template <typename S, int MODE, bool RECORD>
+// HERE: flagged lanes are handed back in *flagged, to be collided in FP64 by the caller.
+template <typename S, int MODE, bool RECORD, bool HERE = false>
 __device__ __forceinline__ void node_update_adj(const S* src, S* dst, const Geo& g, uint32_t x,
                                                 uint32_t y, uint32_t z, const CollideParams& cp,
-                                                float* gamma_out, StepCounters* ctr) {
+                                                float* gamma_out, StepCounters* ctr,
+                                                int* flagged = nullptr) {
   using C = Codec<S>;
   using Pat = Pattern<MODE>;
   using IO = PairIO<S>;
@@ -1593,7 +1595,9 @@ __device__ __forceinline__ void node_update_adj(const S* src, S* dst, const Geo&
       if (wb) IO::put1(at(plane, o1, o2, x), d[I].y);
     }
   });
-  if (fp64) {
+  if constexpr (HERE) {
+    *flagged = fp64;
+  } else if (fp64) {
     if (fp64 & 1) flag_fp64(g, oy[1] + oz[1] + x);
     if (fp64 & 2) flag_fp64(g, oy[1] + oz[1] + x + 1);
   }

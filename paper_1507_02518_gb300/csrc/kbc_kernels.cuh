@@ -28,10 +28,10 @@ template <> struct MaxThreads<double> { static constexpr int value = 256; };
 // ends. What it hides is the launch latency between kernels and the start of the next one behind
 // the last blocks of this: 32^3 FP32 AA (step and pass) 9.2 -> 5.4 us a step with the node order
 // below, 256^3 pull 542 -> 537 us. Launched without the attribute, follow() does nothing.
-// Where waiting blocks take places that unbalance the next kernel over the SMs, the next one is
-// let in at the end only: the pull step (let_next(): 32^3 3.9 -> 3.4 us, 48^3 5.2 -> 4.9; the AA
-// step is better with follow(), 4.4 against 4.7), and the FP64 step, whose blocks fill an SM with
-// three, when they exit (32^3 11.2 -> 8.7 us).
+// Blocks that wait on an SM take places there and unbalance the next kernel over the SMs, so the
+// adjacent-pair steps let the next kernel in at their end only (let_next(): 32^3 FP32 pull 3.9 ->
+// 3.4 us, AA without a pass 4.6 -> 3.2), and the FP64 step, whose blocks fill an SM with three, when
+// its blocks exit (32^3 11.2 -> 8.7 us).
 __device__ __forceinline__ void wait_before() { cudaGridDependencySynchronize(); }
 __device__ __forceinline__ void let_next() { cudaTriggerProgrammaticLaunchCompletion(); }
 __device__ __forceinline__ void follow() {
@@ -151,7 +151,6 @@ template <typename S, int MODE, bool RECORD, bool AHEAD>
 __global__ void __launch_bounds__(128, 3) adj_step_kernel(const S* src, S* dst, Geo g,
                                                        CollideParams cp, float* gamma_out,
                                                        StepCounters* ctr) {
-  if (MODE != MODE_PULL) let_next();
   wait_before();
   if constexpr (AHEAD)
     prefetch_ahead<S>(src, g, (uint64_t)(blockIdx.z + g.zb) * g.nxy +
@@ -160,7 +159,7 @@ __global__ void __launch_bounds__(128, 3) adj_step_kernel(const S* src, S* dst, 
   if (x >= g.nx) return;
   node_update_adj<S, MODE, RECORD>(src, dst, g, x, blockIdx.y, blockIdx.z + g.zb, cp,
                                    gamma_out, ctr);
-  if (MODE == MODE_PULL) let_next();
+  let_next();
 }
 
 // The same over the box's node order: pair k is nodes (2k, 2k + 1), which share a row as nx is
@@ -171,7 +170,6 @@ template <typename S, int MODE, bool RECORD, bool AHEAD>
 __global__ void __launch_bounds__(128, 3) adj_linear_kernel(const S* src, S* dst, Geo g,
                                                          CollideParams cp, float* gamma_out,
                                                          StepCounters* ctr) {
-  if (MODE != MODE_PULL) let_next();
   wait_before();
   const uint32_t n = g.zb * g.nxy + 2 * (blockIdx.x * blockDim.x + threadIdx.x);  // P < 2^31
   if (n >= g.ze * g.nxy) return;
@@ -180,14 +178,65 @@ __global__ void __launch_bounds__(128, 3) adj_linear_kernel(const S* src, S* dst
   const uint32_t z = row / g.ny;
   node_update_adj<S, MODE, RECORD>(src, dst, g, n - row * g.nx, row - z * g.ny, z, cp, gamma_out,
                                    ctr);
-  if (MODE == MODE_PULL) let_next();
+  let_next();
+}
+
+// The adjacent-pair FP32 step of a small box, over the node order, with the FP64 re-collision in the
+// kernel instead of in a pass after it: the launch of the pass costs as much as the step there.
+// node_update_adj<..., true> hands back the flagged lanes (their FP32 results are stored by the pull
+// step, not by AA); a lane's FP64 collision needs its own inputs only, which are still in place.
+// Rule: up to 2^18 nodes. us a step with the pass -> without: FP32 pull 16^3 3.5 -> 2.6 (the rate at
+// which the host launches), 32^3 3.6 -> 2.7, 48^3 5.1 -> 4.2, 64^3 9.0 -> 8.3, AA 32^3 5.2 -> 3.2, 64^3
+// 9.6 -> 9.3; beyond, the call in the step kernel costs more than the pass (128^3 AA 69.8 -> 77.3).
+constexpr uint64_t kSmallNodes = 1ull << 18;
+template <int MODE>
+__device__ __noinline__ void recollide_here(const float* src, float* dst, Geo g, uint32_t n,
+                                            CollideParams cp, float* gamma_out,
+                                            StepCounters* ctr) {
+  const uint32_t row = n / g.nx, z = row / g.ny;
+  int gd = 0;
+  const float gam = fix_node_update<float, MODE>(src, dst, g, n - row * g.nx, row - z * g.ny, z, cp,
+                                                 &gd);
+  if (gamma_out) {
+    gamma_out[n] = gam;
+    if (gd) atomicAdd(&ctr->guarded, 1ull);
+  }
+}
+template <int MODE, bool RECORD>
+__global__ void __launch_bounds__(128, 3) adj_small_kernel(const float* src, float* dst, Geo g,
+                                                        CollideParams cp, float* gamma_out,
+                                                        StepCounters* ctr) {
+  wait_before();
+  const uint32_t n = g.zb * g.nxy + 2 * (blockIdx.x * blockDim.x + threadIdx.x);  // P < 2^31
+  if (n >= g.ze * g.nxy) return;
+  const uint32_t row = n / g.nx;
+  const uint32_t z = row / g.ny;
+  int flagged = 0;
+  node_update_adj<float, MODE, RECORD, true>(src, dst, g, n - row * g.nx, row - z * g.ny, z, cp,
+                                             gamma_out, ctr, &flagged);
+  if (flagged & 1) recollide_here<MODE>(src, dst, g, n, cp, RECORD ? gamma_out : nullptr, ctr);
+  if (flagged & 2) recollide_here<MODE>(src, dst, g, n + 1, cp, RECORD ? gamma_out : nullptr, ctr);
+  let_next();
+}
+// whether the step of this box re-collides its flagged nodes itself (no pass follows)
+template <typename S, bool CENTRAL, bool POLY>
+inline bool small_step(const Geo& g, const CollideParams& cp, const StepOpts& o) {
+  return std::is_same<S, float>::value && !CENTRAL && !POLY && g.nx % 2 == 0 && g.P <= kSmallNodes &&
+         cp.gamma_mode == GAMMA_ESTIMATE && (o.kernel == KERNEL_ADJ || o.kernel == KERNEL_AUTO);
 }
 
 // Rows of a multiple of 64 nodes: blocks of whole row segments; other rows: the node order.
 template <typename S, int MODE, bool RECORD>
 static cudaError_t launch_adj(const S* src, S* dst, const Geo& g, const CollideParams& cp,
-                              float* gamma_out, StepCounters* ctr, cudaStream_t st) {
+                              float* gamma_out, StepCounters* ctr, bool small, cudaStream_t st) {
   const uint32_t pairs = g.nx / 2;
+  if constexpr (std::is_same<S, float>::value) {
+    if (small) {
+      const uint32_t all = pairs * g.ny * (g.ze - g.zb);
+      return launch_following(adj_small_kernel<MODE, RECORD>, (all + 127) / 128, 128, st, src, dst,
+                              g, cp, gamma_out, ctr);
+    }
+  }
   auto run = [&](auto ahead) {
     constexpr bool A = decltype(ahead)::value;
     if (pairs % 32 != 0) {
@@ -574,7 +623,8 @@ static cudaError_t launch_step_c(const BoxView& b, const S* src, S* dst, const G
       // the default for even rows: adjacent pairs (measured faster than (x, x + 32) pairs at
       // 256^3: FP32 AA 0.549 vs 0.630 ms, FP16 AA 0.446 vs 0.504 ms, pull equal or better)
       if ((o.kernel == KERNEL_ADJ || o.kernel == KERNEL_AUTO) && g.nx % 2 == 0)
-        return launch_adj<S, MODE, RECORD>(src, dst, g, cp, b.gamma, ctr, st);
+        return launch_adj<S, MODE, RECORD>(src, dst, g, cp, b.gamma, ctr,
+                                           small_step<S, CENTRAL, POLY>(g, cp, o), st);
     }
     if (o.kernel == KERNEL_PACKED || o.kernel == KERNEL_AUTO || o.kernel == KERNEL_ROWS)
       return launch_pair<S, MODE, RECORD, CENTRAL, POLY>(src, dst, g, cp, b.gamma, ctr, st);
@@ -600,7 +650,8 @@ static cudaError_t launch_step_p(const BoxView& b, const S* src, S* dst, const G
                                  cudaStream_t st) {
   cudaError_t e = launch_step_c<S, MODE, RECORD, CENTRAL, POLY>(b, src, dst, g, cp, o, ctr, st);
   if constexpr (std::is_same<S, float>::value) {
-    if (e == cudaSuccess && cp.gamma_mode == GAMMA_ESTIMATE) {
+    if (e == cudaSuccess && cp.gamma_mode == GAMMA_ESTIMATE &&
+        !small_step<S, CENTRAL, POLY>(g, cp, o)) {
       const uint64_t warps = (g.P + 1023) / 1024;  // a warp takes 32 mask words
       uint64_t blocks = (32 * warps + kPassThreads - 1) / kPassThreads;
       if (blocks > (uint64_t)kPassBlocks) blocks = kPassBlocks;
