@@ -485,6 +485,53 @@ __device__ __forceinline__ bool near_root(const double (&dh)[27], const double (
   return done;
 }
 
+// The same in FP32: terms to X^12 (2^-25 of the sum at |X| = 1/4), steps until less than 2^-24 of
+// 1 + |gamma| is left. The linear term is summed too (N holds all of g): the estimate is rounded
+// to FP32, and so is its zero. 128^3: 0.387 -> 0.196 ms a step.
+__device__ __forceinline__ bool near_root(const float (&dh)[27], const float (&av)[27],
+                                          const float (&rx)[3], const float (&ry)[3],
+                                          const float (&rz)[3], float beta, float den,
+                                          float* gamma) {
+  float d = 0.0f;
+#pragma unroll 1
+  for (int it = 0; it < 4; ++it) {
+    const float bg = -fmaf(beta, *gamma, d);
+    float N = 0.0f, d1 = 0.0f, d2 = 0.0f, top = 0.0f;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        const float ryz = ry[b] * rz[c];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          const int i = a + 3 * b + 9 * c;
+          const float r = rx[a] * ryz, X = fmaf(bg, dh[i], av[i]) * r;
+          top = fmaxf(top, fabsf(X));
+          float q = -1.0f / 12.0f;
+#pragma unroll
+          for (int m = 11; m >= 2; --m) q = fmaf(X, q, (m & 1 ? 1.0f : -1.0f) / (float)m);
+          const float hx = dh[i] * X, y = dh[i] * r, v = rcp_approx(1.0f + X);
+          N = fmaf(hx, fmaf(X, q, 1.0f), N);
+          d1 = fmaf(hx * r, dh[i] * v, d1);
+          d2 = fmaf(dh[i] * y, y * (v * v), d2);
+        }
+      }
+    }
+    const float slope = den - d1;
+    if (!(top < 0.25f) || !(slope > 0.25f * den)) return false;
+    const float ir = rcp_approx(slope);
+    float st = N * ir;
+    if (it == 0) st = (N - 0.5f * d2 * st * st) * ir;
+    d += st;
+    const float left = fabsf(st) * (1e-5f + fabsf(st * d2) * ir);
+    if (left <= 6e-8f) {
+      *gamma += d / beta;
+      return true;
+    }
+  }
+  return false;
+}
+
 // One KBC collision on the shifted populations d[i] = f_i - W_i, in place: the post-collision
 // state of eq:Egeneral with the mirror state eq:ksh-mirror, f' = f - beta (2 ds + gamma dh),
 // ds = s - s_eq by Table 1, dh = f - f_eq - ds, gamma by eq:result21 (Sec. KBC); R holds one
@@ -858,9 +905,7 @@ __device__ __forceinline__ R collide(R (&d)[27], const CollideParams& cp, int* g
     int status = 1;
     // guarded (<dh|dh> ~ 0) and non-finite nodes keep the estimate's value
     if (!gmask && gamma == gamma && cp.gamma_mode == GAMMA_EXACT) {
-      if constexpr (std::is_same<T, double>::value) {
-        if (near_root(dh, av, rx, ry, rz, cp.beta, den, &gamma)) status = 0;
-      }
+      if (near_root(dh, av, rx, ry, rz, prec<T>(cp.beta, cp.betaf), den, &gamma)) status = 0;
       if (status != 0)
         gamma = newton_gamma<T>(dh, av, rx, ry, rz, prec<T>(cp.beta, cp.betaf), gamma, &status);
     }
