@@ -20,32 +20,63 @@ constexpr size_t kAlign = 256;
 
 size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 
-template <typename C> __device__ __forceinline__ double norm2(const C& c) {
-  return (double)c.x * (double)c.x + (double)c.y * (double)c.y;
+// FP32 to FP64 by the bits (a conversion costs the FP64 pipe as much as an FMA)
+__device__ __forceinline__ double widen(float v) {
+  const uint32_t b = __float_as_uint(v), a = b & 0x7fffffffu;
+  if (a - 0x00800000u >= 0x7f000000u) return (double)v;  // zero, subnormal, infinite, NaN
+  return __hiloint2double((int)((b & 0x80000000u) | ((a >> 3) + 0x38000000u)), (int)(b << 29));
+}
+__device__ __forceinline__ double norm2(const cufftComplex& c) {
+  const double x = widen(c.x), y = widen(c.y);
+  return __fma_rn(x, x, __dmul_rn(y, y));
+}
+__device__ __forceinline__ double norm2(const cufftDoubleComplex& c) {
+  return __fma_rn(c.x, c.x, __dmul_rn(c.y, c.y));
 }
 
+// A warp takes 32 consecutive kx of a row (ky, kz): their shells do not decrease, so modes of the
+// same shell are neighbours, and the warp adds them up before one lane of each run adds to the
+// histogram (an FP64 addition in shared memory is a compare-and-swap loop, which the modes of a
+// row near kx = 0 all wanted at once). The shell is exact in integers: the FP32 square root is
+// corrected by 4 k^2 against (2m +- 1)^2. 256^3 FP32
+// spectrum 3.08 -> 2.31 ms (FP64 12.97 -> 7.88), of which 185 us for the shells of a component.
 template <typename C>
 __global__ void __launch_bounds__(256) shell_kernel(const C* X, uint32_t n, int nbins,
                                                     double scale, double* partials) {
   extern __shared__ double hist[];
   for (int m = threadIdx.x; m < nbins; m += blockDim.x) hist[m] = 0.0;
   __syncthreads();
-  const uint32_t nh = n / 2 + 1;
-  const uint64_t total = (uint64_t)n * n * nh;
-  for (uint64_t idx = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; idx < total;
-       idx += (uint64_t)gridDim.x * blockDim.x) {
-    const uint32_t kx = (uint32_t)(idx % nh);
-    const uint64_t r = idx / nh;
-    const uint32_t ky = (uint32_t)(r % n), kz = (uint32_t)(r / n);
-    const int ix = (int)kx;
+  const uint32_t nh = n / 2 + 1, chunks = (nh + 31) / 32, lane = threadIdx.x & 31;
+  const uint32_t units = n * n * chunks;  // n^3 < 2^31
+  const uint32_t warps = gridDim.x * (blockDim.x >> 5);
+  for (uint32_t q = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); q < units; q += warps) {
+    const uint32_t row = q / chunks, kx = (q - row * chunks) * 32 + lane;
+    const uint32_t kz = row / n, ky = row - kz * n;
     const int iy = ky <= n / 2 ? (int)ky : (int)ky - (int)n;
     const int iz = kz <= n / 2 ? (int)kz : (int)kz - (int)n;
-    if (ix == 0 && iy == 0 && iz == 0) continue;
-    // the half spectrum holds one of each pair (n, -n), whose two halves |u_hat|^2 / 2 are
-    // equal, except on the kx = 0 and kx = n/2 planes, which hold both members
-    const double w = (kx == 0 || (n % 2 == 0 && kx == n / 2)) ? 1.0 : 2.0;
-    const int m = (int)rint(sqrt((double)(ix * ix + iy * iy + iz * iz)));
-    if (m < nbins) atomicAdd(&hist[m], w * scale * norm2(X[idx]));
+    double v = 0.0;
+    int m = 0x7fffffff;  // lanes without a mode: a run of their own
+    if (kx < nh) {
+      const int k2 = (int)kx * (int)kx + iy * iy + iz * iz;
+      m = (int)(sqrtf((float)k2) + 0.5f);
+      if (4 * k2 > (2 * m + 1) * (2 * m + 1)) ++m;
+      else if (m > 0 && 4 * k2 < (2 * m - 1) * (2 * m - 1)) --m;
+      // the half spectrum holds one of each pair (n, -n), whose two halves |u_hat|^2 / 2 are
+      // equal, except on the kx = 0 and kx = n/2 planes, which hold both members
+      const double w = (kx == 0 || (n % 2 == 0 && kx == n / 2)) ? scale : 2.0 * scale;
+      v = __dmul_rn(w, norm2(X[(uint64_t)row * nh + kx]));
+      if (k2 == 0) m = -1;  // the mean flow is left out
+    }
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int mm = __shfl_down_sync(0xffffffffu, m, o);
+      const bool same = lane + o < 32 && mm == m;
+      if (!__any_sync(0xffffffffu, same)) break;
+      const double add = __shfl_down_sync(0xffffffffu, v, o);
+      if (same) v = __dadd_rn(v, add);
+    }
+    const int before = __shfl_up_sync(0xffffffffu, m, 1);
+    if ((lane == 0 || before != m) && m >= 0 && m < nbins) atomicAdd(&hist[m], v);
   }
   __syncthreads();
   for (int m = threadIdx.x; m < nbins; m += blockDim.x)
