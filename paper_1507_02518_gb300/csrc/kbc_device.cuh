@@ -404,6 +404,12 @@ __device__ __forceinline__ double long_of(float v) {
       a < 0x00800000u ? 0 : (int)((b & 0x80000000u) | ((a >> 3) + 0x38000000u)), (int)(b << 29));
 }
 
+// short_of() rounded to nearest (the carry may run into the exponent)
+__device__ __forceinline__ float near_of(double v) {
+  const float t = short_of(v);
+  return __uint_as_float(__float_as_uint(t) + (((uint32_t)__double2loint(v) >> 28) & 1u));
+}
+
 // The FP64 root gamma* of eq:result1 near the estimate g0, for nodes not far from equilibrium.
 // With X_i = (a_i - beta gamma dh_i) / f_eq_i, the estimate solves sum dh_i X_i = 0, so that at
 // gamma = g0 + d / beta
@@ -411,25 +417,70 @@ __device__ __forceinline__ double long_of(float v) {
 // and the root d = N(d) / den is a small number: N needs 2^-44 of itself where newton_gamma()
 // needs g to 2^-53 of its terms. ln(1 + X) - X = X^2 (-1/2 + X/3 - X^2/4 + ...) for |X| < 1/4: terms
 // to X^12 in FP64, those to X^22 in FP32 (together 2^-44 of the sum at 1/4, less below); the
-// derivatives by d in FP32. A step of fourth order at d = 0, then Newton steps until the error
-// they leave (the FP32 slope's and the curvature's share) is below 2^-53: one, seldom two. 18
-// FP64 operations per population and evaluation and two evaluations; newton_gamma() takes four
-// with a log1p and a division each. False (gamma untouched) when some |X| is 1/4 or more or the
-// steps do not converge. 96^3: 7.93 -> 2.60 ms a step, the gap 8.16 -> 2.67;
-// the collision itself takes 0.9 of that on the FP64 pipe.
+// derivatives by d in FP32. FP32 evaluations alone (near_start()) first take d to a few 1e-9; an
+// FP64 one then takes it to half an ulp of gamma = 2, seldom a second: the error left is the step
+// times what the FP32 slope and curvature may be off. 17 FP64 operations per population and evaluation,
+// where newton_gamma() takes four evaluations with a log1p and a division each. False (gamma
+// untouched) when some |X| is 1/4 or more or the steps do not converge. 96^3: 7.93 -> 2.08 ms a
+// step (2.60 with the first steps in FP64 too); the collision itself takes 0.9 of that on the FP64
+// pipe.
+__device__ __forceinline__ bool near_start(const double (&dh)[27], const double (&av)[27],
+                                           const double (&rx)[3], const double (&ry)[3],
+                                           const double (&rz)[3], float beta_gamma, float den,
+                                           float* start) {
+  float d = 0.0f;
+  const float sx[3] = {near_of(rx[0]), near_of(rx[1]), near_of(rx[2])};
+#pragma unroll 1
+  for (int it = 0; it < 4; ++it) {
+    const float bg = -(beta_gamma + d);
+    float N = 0.0f, d1 = 0.0f, d2 = 0.0f, top = 0.0f;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        const float ryz = near_of(ry[b]) * near_of(rz[c]);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          const int i = a + 3 * b + 9 * c;
+          const float hf = near_of(dh[i]), r = sx[a] * ryz;
+          const float X = fmaf(bg, hf, near_of(av[i])) * r;
+          top = fmaxf(top, fabsf(X));
+          float q = -1.0f / 12.0f;
+#pragma unroll
+          for (int m = 11; m >= 2; --m) q = fmaf(X, q, (m & 1 ? 1.0f : -1.0f) / (float)m);
+          const float hx = hf * X, y = hf * r, v = rcp_approx(1.0f + X);
+          N = fmaf(hx, X * q, N);
+          d1 = fmaf(hx * r, hf * v, d1);
+          d2 = fmaf(hf * y, y * (v * v), d2);
+        }
+      }
+    }
+    const float slope = den - d1;
+    if (!(top < 0.25f) || !(slope > 0.25f * den)) return false;
+    const float h = fmaf(-d, den, N), ir = rcp_approx(slope);
+    float st = h * ir;
+    st = (h - 0.5f * d2 * st * st) * ir;
+    d += st;
+    if (fabsf(st) < 5e-4f) break;
+  }
+  *start = d;
+  return true;
+}
+
 __device__ __forceinline__ bool near_root(const double (&dh)[27], const double (&av)[27],
                                           const double (&rx)[3], const double (&ry)[3],
                                           const double (&rz)[3], double beta, double den,
                                           double* gamma) {
   const float df = short_of(den);
-  double d = 0.0;
-  bool done = false;
-  if (!(df > 0.0f)) return false;
+  float start;
+  if (!(df > 0.0f) || !near_start(dh, av, rx, ry, rz, short_of(__dmul_rn(beta, *gamma)), df, &start))
+    return false;
+  double d = long_of(start);
 #pragma unroll 1
-  for (int it = 0; it < 5; ++it) {
+  for (int it = 0; it < 4; ++it) {
     const double bg = -__fma_rn(beta, *gamma, d);
     double N = 0.0;
-    float d1 = 0.0f, d2 = 0.0f, d3 = 0.0f;
+    float d1 = 0.0f, d2 = 0.0f;
     uint32_t top = 0;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -455,34 +506,29 @@ __device__ __forceinline__ bool near_root(const double (&dh)[27], const double (
           const float v = rcp_approx(1.0f + xf);
           d1 = fmaf(hf * y, xf * v, d1);
           d2 = fmaf(hf * y, y * (v * v), d2);
-          d3 = fmaf(hf * y, (y * v) * (y * v) * (v + v), d3);
         }
       }
     }
-    // h(d) = N - d den, h' = -(den - d1), h'' = -d2, h''' = -d3
+    // h(d) = N - d den, h' = -(den - d1), h'' = -d2
     const double slope = __dadd_rn(den, -long_of(d1));
-    if (top >= 0x3fd00000u || !(short_of(slope) > 0.25f * df)) break;
+    if (top >= 0x3fd00000u || !(short_of(slope) > 0.25f * df)) return false;
     const double h = __fma_rn(-d, den, N);
     double ir = long_of(rcp_approx(short_of(slope)));
     ir = __fma_rn(ir, __fma_rn(-slope, ir, 1.0), ir);
-    double st = __dmul_rn(h, ir);
-    if (it == 0) {
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        const float x = short_of(st);
-        st = __dmul_rn(h - long_of(x * x * (0.5f * d2 + x * d3 * (1.0f / 6.0f))), ir);
-      }
-    }
+    const float irf = short_of(ir), s1 = short_of(__dmul_rn(h, ir));
+    const double st = __dmul_rn(h - long_of(0.5f * d2 * s1 * s1), ir);
     d = __dadd_rn(d, st);
-    // what a Newton step leaves: its share of the slope's FP32 error and of the curvature
-    const float sf = fabsf(short_of(st));
-    if (it > 0 && sf * (1e-7f + fabsf(sf * d2) * short_of(ir)) <= 1e-16f) {
-      done = true;
-      break;
+    // what the step leaves: the slope's FP32 error (d1 <= max|X| den), the curvature's and the
+    // third order's
+    const float sf = fabsf(short_of(st)), q = sf * d2 * irf;
+    const float xm = __uint_as_float((top - 0x38000000u) << 3);  // max |X|
+    const float off = 2e-7f * (top > 0x38800000u ? xm : 1e-30f) * df * irf;
+    if (sf * (off + q * (1e-6f + 2.0f * q)) <= 2e-16f) {
+      *gamma = *gamma + d / beta;
+      return true;
     }
   }
-  if (done) *gamma = *gamma + d / beta;
-  return done;
+  return false;
 }
 
 // The same in FP32: terms to X^12 (2^-25 of the sum at |X| = 1/4), steps until less than 2^-24 of
