@@ -26,20 +26,23 @@ __device__ __forceinline__ double widen(float v) {
   if (a - 0x00800000u >= 0x7f000000u) return (double)v;  // zero, subnormal, infinite, NaN
   return __hiloint2double((int)((b & 0x80000000u) | ((a >> 3) + 0x38000000u)), (int)(b << 29));
 }
-__device__ __forceinline__ double norm2(const cufftComplex& c) {
+// |c|^2 + sum
+__device__ __forceinline__ double norm2(const cufftComplex& c, double sum) {
   const double x = widen(c.x), y = widen(c.y);
-  return __fma_rn(x, x, __dmul_rn(y, y));
+  return __fma_rn(x, x, __fma_rn(y, y, sum));
 }
-__device__ __forceinline__ double norm2(const cufftDoubleComplex& c) {
-  return __fma_rn(c.x, c.x, __dmul_rn(c.y, c.y));
+__device__ __forceinline__ double norm2(const cufftDoubleComplex& c, double sum) {
+  return __fma_rn(c.x, c.x, __fma_rn(c.y, c.y, sum));
 }
 
-// A warp takes 32 consecutive kx of a row (ky, kz): their shells do not decrease, so modes of the
-// same shell are neighbours, and the warp adds them up before one lane of each run adds to the
+// A warp takes 32 consecutive kx of the up to four rows (+-ky, +-kz), whose modes lie on the same
+// shells: a lane adds its four modes by FMAs (FP64 additions bound this kernel: 3.5 FP64
+// instructions a mode, 9 for one row at a time, 185 us). Along kx the shells do not decrease, so
+// modes of the same shell are neighbours, and the warp adds them up before one lane of each run adds to the
 // histogram (an FP64 addition in shared memory is a compare-and-swap loop, which the modes of a
 // row near kx = 0 all wanted at once). The shell is exact in integers: the FP32 square root is
 // corrected by 4 k^2 against (2m +- 1)^2. 256^3 FP32
-// spectrum 3.08 -> 2.31 ms (FP64 12.97 -> 7.88), of which 185 us for the shells of a component.
+// spectrum 3.08 -> 2.07 ms (FP64 12.97 -> 7.66), the shells of a component 355 -> 110 us.
 template <typename C>
 __global__ void __launch_bounds__(256) shell_kernel(const C* X, uint32_t n, int nbins,
                                                     double scale, double* partials) {
@@ -47,24 +50,28 @@ __global__ void __launch_bounds__(256) shell_kernel(const C* X, uint32_t n, int 
   for (int m = threadIdx.x; m < nbins; m += blockDim.x) hist[m] = 0.0;
   __syncthreads();
   const uint32_t nh = n / 2 + 1, chunks = (nh + 31) / 32, lane = threadIdx.x & 31;
-  const uint32_t units = n * n * chunks;  // n^3 < 2^31
+  const uint32_t units = nh * nh * chunks;
   const uint32_t warps = gridDim.x * (blockDim.x >> 5);
   for (uint32_t q = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); q < units; q += warps) {
     const uint32_t row = q / chunks, kx = (q - row * chunks) * 32 + lane;
-    const uint32_t kz = row / n, ky = row - kz * n;
-    const int iy = ky <= n / 2 ? (int)ky : (int)ky - (int)n;
-    const int iz = kz <= n / 2 ? (int)kz : (int)kz - (int)n;
+    const uint32_t kz = row / nh, ky = row - kz * nh;
+    // the rows n - ky and n - kz, where they are rows of their own
+    const bool my = ky != 0 && 2 * ky != n, mz = kz != 0 && 2 * kz != n;
     double v = 0.0;
     int m = 0x7fffffff;  // lanes without a mode: a run of their own
     if (kx < nh) {
-      const int k2 = (int)kx * (int)kx + iy * iy + iz * iz;
+      const int k2 = (int)(kx * kx + ky * ky + kz * kz);
       m = (int)(sqrtf((float)k2) + 0.5f);
       if (4 * k2 > (2 * m + 1) * (2 * m + 1)) ++m;
       else if (m > 0 && 4 * k2 < (2 * m - 1) * (2 * m - 1)) --m;
+      auto at = [&](uint32_t y, uint32_t z) { return X[((uint64_t)z * n + y) * nh + kx]; };
+      v = norm2(at(ky, kz), 0.0);
+      if (my) v = norm2(at(n - ky, kz), v);
+      if (mz) v = norm2(at(ky, n - kz), v);
+      if (my && mz) v = norm2(at(n - ky, n - kz), v);
       // the half spectrum holds one of each pair (n, -n), whose two halves |u_hat|^2 / 2 are
       // equal, except on the kx = 0 and kx = n/2 planes, which hold both members
-      const double w = (kx == 0 || (n % 2 == 0 && kx == n / 2)) ? scale : 2.0 * scale;
-      v = __dmul_rn(w, norm2(X[(uint64_t)row * nh + kx]));
+      v = __dmul_rn(v, (kx == 0 || (n % 2 == 0 && kx == n / 2)) ? scale : 2.0 * scale);
       if (k2 == 0) m = -1;  // the mean flow is left out
     }
 #pragma unroll
