@@ -167,27 +167,61 @@ template <int N> KBC_HD double to_f64(fx v) {
   return f64_of((uint64_t)hi << 32 | (uint32_t)b);
 }
 
-// v * 2^-(60 + n) in FP32: rounded to nearest even, or towards zero with the lost bits in the
-// last one (round to odd: a further rounding to a shorter type is then the only one)
-KBC_HD float i2f(uint32_t x) { return (float)x; }
+// a 2^-n + b, n < 64, rounded to nearest or towards zero (a and b exact)
+template <int N> KBC_HD float add_rn(float a, float b) {
+  constexpr float c = 1.0f / (float)(1ull << N);
+#ifdef __CUDA_ARCH__
+  return __fmaf_rn(a, c, b);
+#else
+  return fmaf(a, c, b);
+#endif
+}
+template <int N> KBC_HD float add_rz(float a, float b) {
+  constexpr float c = 1.0f / (float)(1ull << N);
+#ifdef __CUDA_ARCH__
+  return __fmaf_rz(a, c, b);
+#else
+  const double s = (double)a * c + (double)b;  // exact: 48 bits
+  const float f = (float)s;
+  return fabs((double)f) > fabs(s) ? f32_of(bits_of(f) - 1) : f;
+#endif
+}
+// 24 bits of v from bit S on, as a float
+template <int S> KBC_HD float window(fx v, uint32_t sticky) {
+  return (float)(int32_t)(((uint32_t)((uint64_t)v >> S) & 0xffffffu) | sticky);
+}
+
+// v * 2^-(60 + N) in FP32, rounded to nearest even. The short way, for 2^38 <= |v| < 2^60: the sum
+// of bits 36 and above and of the 24 below, both exact in FP32, is rounded once; the last 12 bits
+// count as a sticky bit, two places below the rounding one. Less than that is normalised first
+// (that way for every value took 36 of the 57 instructions a population of an FP32
+// initialisation: 256^3 1.00 -> 0.80 ms).
+KBC_HD bool short_way(fx v) { return (uint32_t)((int32_t)((uint64_t)v >> 32) + 64) >= 128u; }
+template <int N> KBC_HD float to_f32_short(fx v) {
+  return add_rn<24 + N>((float)((int32_t)((uint64_t)v >> 32) >> 4),
+                        mulf(window<12>(v, ((uint32_t)v & 0xfffu) != 0),
+                             1.0f / (float)(1ull << (48 + N))));
+}
 template <int N> KBC_HD float to_f32(fx v) {
+  if (short_way(v)) return to_f32_short<N>(v);
   const uint64_t a = v < 0 ? 0 - (uint64_t)v : (uint64_t)v;
   const int lz = clz64(a);
   const uint64_t q = lz == 64 ? 0 : a << lz;
   // the leading 32 bits, the rest as a sticky bit: the conversion rounds at bit 24
   const uint32_t t = (uint32_t)(q >> 32) | ((uint32_t)q != 0 ? 1u : 0u);
-  const uint32_t b = bits_of(i2f(t));  // t 2^(32 - lz) of the units
+  const uint32_t b = bits_of((float)t);  // t 2^(32 - lz) of the units
   const uint32_t r = t == 0 ? 0 : b + ((uint32_t)(32 - kFrac - N - lz) << 23);
   return f32_of(r | ((uint32_t)((uint64_t)v >> 32) & 0x80000000u));
 }
+// The same towards zero with the last bit set (0 stays 0), for a further rounding to a shorter
+// type, which then rounds v (a tie of it away from zero) as long as it has at most 22 bits of v
+// from 2^16 units, 2^-44, on. |v| < 2^63. FP16 initialisation of 256^3: 1.08 -> 0.79 ms.
 template <int N> KBC_HD float to_f32_odd(fx v) {
-  const uint64_t a = v < 0 ? 0 - (uint64_t)v : (uint64_t)v;
-  const int lz = clz64(a);
-  const uint64_t q = lz == 64 ? 0 : a << lz;
-  const uint32_t t = (uint32_t)(q >> 40) | ((q << 24) != 0 ? 1u : 0u);  // 24 bits: exact
-  const uint32_t b = bits_of(i2f(t));
-  const uint32_t r = t == 0 ? 0 : b + ((uint32_t)(40 - kFrac - N - lz) << 23);
-  return f32_of(r | ((uint32_t)((uint64_t)v >> 32) & 0x80000000u));
+  const int32_t hi = (int32_t)((uint64_t)v >> 32);
+  const float f = add_rz<20 + N>((float)(hi >> 8),
+                                 mulf(window<16>(v, ((uint32_t)v & 0xffffu) != 0),
+                                      1.0f / (float)(1ull << (44 + N))));
+  return f32_of(bits_of(f) | (v != 0 ? 1u : 0u));
 }
 
 // ------------------------------------------------------------------ products

@@ -38,11 +38,11 @@ __device__ __forceinline__ double norm2(const cufftDoubleComplex& c, double sum)
 // A warp takes 32 consecutive kx of the up to four rows (+-ky, +-kz), whose modes lie on the same
 // shells: a lane adds its four modes by FMAs (FP64 additions bound this kernel: 3.5 FP64
 // instructions a mode, 9 for one row at a time, 185 us). Along kx the shells do not decrease, so
-// modes of the same shell are neighbours, and the warp adds them up before one lane of each run adds to the
-// histogram (an FP64 addition in shared memory is a compare-and-swap loop, which the modes of a
-// row near kx = 0 all wanted at once). The shell is exact in integers: the FP32 square root is
-// corrected by 4 k^2 against (2m +- 1)^2. 256^3 FP32
-// spectrum 3.08 -> 2.07 ms (FP64 12.97 -> 7.66), the shells of a component 355 -> 110 us.
+// modes of the same shell are neighbours, and the warp adds them up before one lane of each run
+// adds to the histogram (an FP64 addition in shared memory is a compare-and-swap loop, which the
+// modes of a row near kx = 0 all wanted at once). The shell is exact in integers: the FP32 square
+// root is corrected by 4 k^2 against (2m +- 1)^2. 256^3 FP32 spectrum 3.08 -> 2.07 ms (FP64
+// 12.97 -> 7.66), the shells of a component 355 -> 110 us.
 template <typename C>
 __global__ void __launch_bounds__(256) shell_kernel(const C* X, uint32_t n, int nbins,
                                                     double scale, double* partials) {

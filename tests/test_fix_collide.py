@@ -62,6 +62,12 @@ extern "C" void fix_round(int n, const double* d, double* o, const float* f, dou
     of[k] = fix::to_f64<0>(fix::from_f32(f[k], &top));
   }
 }
+extern "C" void fix_to_f32(int n, const long long* v, float* f, float* odd) {
+  for (int k = 0; k < n; ++k) {
+    f[k] = fix::to_f32<2>(v[k]);
+    odd[k] = fix::to_f32_odd<2>(v[k]);
+  }
+}
 '''
 
 
@@ -235,3 +241,24 @@ def test_equilibrium_and_its_roundings(lib):
     # o is exact here for |v| < 2^53 units and rounded above; FP32 of either is the same
     assert np.array_equal(of, o.astype(np.float32))
     assert np.array_equal(odd.astype(np.float16), o.astype(np.float16))
+
+
+@pytest.mark.parametrize("k", range(14, 60))
+def test_rounding_of_one_binade(lib, k):
+    """FP32 and FP16 of values below 2^k units: ties of FP32 and their neighbours, and the small
+    values next to the bound of the short way (2^38). Exact: one rounding, to nearest even."""
+    rng = np.random.default_rng(k)
+    m = rng.integers(2 ** 24, 2 ** 25, 500)                      # 25 bits: odd ones are ties
+    v = np.concatenate([(m << max(k - 25, 0)) >> max(25 - k, 0), 2 ** k - np.arange(1, 40),
+                        rng.integers(0, 2 ** k, 500)])
+    v = np.concatenate([v - 1, v, v + 1])
+    v = np.concatenate([v, -v])
+    v = np.ascontiguousarray(v[np.abs(v) < 2 ** 60], dtype=np.int64)
+    f, odd = np.empty(len(v), np.float32), np.empty(len(v), np.float32)
+    lib.fix_to_f32(len(v), *[a.ctypes.data_as(ctypes.c_void_p) for a in (v, f, odd)])
+    x = v.astype(LD) * LD(2.0) ** -62
+    assert np.array_equal(f, x.astype(np.float32))
+    # FP16, where it is not a tie: the nearest of the exact value
+    h = odd.astype(np.float16).astype(LD)
+    step = np.maximum(LD(2.0) ** -24, LD(2.0) ** (np.floor(np.log2(np.maximum(np.abs(x), LD(1e-30)))) - 10))
+    assert (np.abs(h - x) <= step / 2).all()
