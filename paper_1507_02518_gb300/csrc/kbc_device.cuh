@@ -3,7 +3,8 @@
 // Method: arXiv:1507.02518, Sec. KBC (eq:Egeneral with eq:ksh-mirror, Table 1, eq:result21) with the
 // product-form equilibrium eq:entropic_eq and the natural moments eq:natmoments.
 //
-// Register-level design (one thread = one lattice node):
+// Register-level design (one thread = one lattice node; the FP64 collision of the natural
+// moments is in kbc_fix.cuh, in fixed point):
 //   * the 27 populations are held as the shift delta_i = f_i - W_i (storage codec below);
 //   * natural moments come from a factorised x -> y -> z reduction of delta;
 //   * the equilibrium is carried per axis: phi(v) = W_v (1 + e_v) with e_0 = -(R-1),
@@ -206,8 +207,9 @@ template <> struct Guard<float> { static constexpr float den = 1e-30f; };
 // from its inputs (fix_node_update), with the FP64 guard of the oracle. The inputs are still
 // in memory then: the pull step reads src only and stores the flagged node's FP32 outputs
 // anyway (the pass overwrites them), the AA step does not store a flagged node (each AA node
-// alone reads and writes its slots). The step kernels hold no call of the FP64 path, which
-// would cost them registers. FP16 storage takes no FP64 path: its rounding of the stored
+// alone reads and writes its slots). The step kernels of large boxes hold no call of the FP64
+// path, which would cost them registers (4 to 18 % of their time); adj_small_kernel does, where
+// the pass's launch costs more. FP16 storage takes no FP64 path: its rounding of the stored
 // populations (the step's output) exceeds the FP32 error of gamma near equilibrium. The
 // FP32 dh carries an absolute error of about 1e-8 (relative to W_i): the round-off of the
 // O(0.1) shifts it is the difference of. At <dh|dh> = 1e-13, |dh / W| ~ 3e-7, so the FP32
@@ -971,8 +973,9 @@ __device__ __forceinline__ R collide(R (&d)[27], const CollideParams& cp, int* g
 //     velocities -1, 0, +1 as 1 : 4 : 1 (that is 6 W_v), so the moments come out 216 times
 //     their value; that factor and the 1/W_i of the outputs sit in the constants of Table 1's
 //     class values, and dh/W = h - G - ds/W needs no weight per population;
-//   * the entropic weights 1/f_eq_i are products of one MUFU reciprocal per axis and velocity
-//     component, for REL (W_i/f_eq_i up to a common factor) of factors without a reciprocal;
+//   * the entropic weights 1/f_eq_i (REL: W_i/f_eq_i) are products of one MUFU reciprocal per
+//     axis and velocity component (factors without a reciprocal, from X_+ X_- = X_0^2, are no
+//     faster: FP16 AA 256^3 381 against 378 us a step);
 //   * the q part's switch multiplies three class constants, not the seven third moments;
 //   * 3u^2 reuses 3u, and the first term of each entropic sum is a product, not an FMA on 0.
 template <typename R, bool REL>
@@ -1122,30 +1125,15 @@ __device__ __forceinline__ R collide_lean(R (&d)[27], const CollideParams& cp, i
   fz[0] = O::sub(tez, uz3);
   fz[1] = O::neg(ez);
   fz[2] = O::add(tez, uz3);
-  // entropic weights per axis: 1 / (W_a X_a), for REL W_a / X_a
+  // entropic weights per axis: REL W_a / X_a, otherwise 1 / (W_a X_a)
   R wx[3], wy[3], wz[3];
-  if constexpr (REL) {
-    // up to factors common to an axis, which drop out of gamma's ratio, 1 / X_+- is X_-+ and 1 / X_0 is
-    // X_0 (the product form has X_+ X_- = X_0^2; rho is such a factor too): no reciprocals
-    const R c6 = O::c(1.0 / 6.0);
-    auto axis_w = [&](R te, R u3, R e, R (&w)[3]) {
-      const R b = O::fma(te, c6, c6), u6 = O::mul(u3, c6);
-      w[0] = O::add(b, u6);
-      w[1] = O::fma(O::neg(c23), e, c23);
-      w[2] = O::sub(b, u6);
-    };
-    axis_w(tex, ux3, ex, wx);
-    axis_w(tey, uy3, ey, wy);
-    axis_w(tez, uz3, ez, wz);
-  } else {
-    // (<dh|dh> itself is compared with kDenFp64 here)
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      const R cw = O::c(a == 1 ? 2.0 / 3.0 : 1.0 / 6.0);
-      wx[a] = O::rcp_fast(O::fma(cw, gx[a], cw));
-      wy[a] = O::rcp_fast(O::fma(cw, fy[a], cw));
-      wz[a] = O::rcp_fast(O::fma(cw, fz[a], cw));
-    }
+  for (int a = 0; a < 3; ++a) {
+    const double Wa = a == 1 ? 2.0 / 3.0 : 1.0 / 6.0;
+    const R cw = O::c(REL ? 1.0 / Wa : Wa);
+    wx[a] = O::rcp_fast(O::fma(cw, gx[a], cw));
+    wy[a] = O::rcp_fast(O::fma(cw, fy[a], cw));
+    wz[a] = O::rcp_fast(O::fma(cw, fz[a], cw));
   }
   // X_a Y_b - 1 for the 9 (a, b) pairs, without cancellation
   R Pab[9];

@@ -1,9 +1,10 @@
 // kbc_kernels.cuh -- CUDA kernels of the D3Q27 KBC step and their launchers.
 //
 // Included once per storage type by kbc_f64.cu / kbc_f32.cu / kbc_f16.cu, which instantiate
-// kbc::Ops<S>. Hot path: step_kernel / pair_step_kernel (one fused stream + KBC collide per
-// node, eq:Egeneral) and batch_kernel / batch_pair_kernel (the same update over a work list of
-// boxes). Transfer, diagnostics and pre-solve kernels are in kbc_aux.cuh.
+// kbc::Ops<S>. Hot path: fix_step_kernel (FP64), adj_*_kernel (FP32 and FP16, even nx; with the
+// FP64 re-collision inside for small boxes), pair_*_kernel (odd nx) and step_kernel: one fused
+// stream + KBC collide per node, eq:Egeneral; batch_*_kernel run the same update over a work
+// list of boxes. Transfer, diagnostics and pre-solve kernels are in kbc_aux.cuh.
 #pragma once
 
 #include <type_traits>
