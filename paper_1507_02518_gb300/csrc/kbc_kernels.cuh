@@ -121,9 +121,11 @@ __device__ __forceinline__ void prefetch_ahead(const S* src, const Geo& g, uint6
     if (sizeof(S) == 4 && n + 32 < g.P) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + 32));
   }
 }
-// where it is worth its instructions: populations larger than L2 (129 MB)
+// where it is worth its instructions: populations larger than L2 (129 MB), of up to 40 GB (FP32 AA
+// without -> with: 640^3 9420 -> 9261 us, 704^3 (38 GB) 11977 -> 11841, 768^3 (49 GB) 14666 -> 15012)
 template <typename S> __host__ __device__ inline bool beyond_l2(const Geo& g) {
-  return 27 * g.P * sizeof(S) > (129ull << 20);
+  const uint64_t bytes = 27 * g.P * sizeof(S);
+  return bytes > (129ull << 20) && bytes <= 40000000000ull;
 }
 
 // Two nodes per thread with packed FP32x2 arithmetic: a block of up to 128 threads covers
@@ -136,7 +138,9 @@ __global__ void __launch_bounds__(128, 3) pair_step_kernel(const S* src, S* dst,
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t xa = blockIdx.x * (2 * blockDim.x) + warp * 64 + lane;
   if (xa >= g.nx) return;
-  if (beyond_l2<S>(g))
+  // FP32 pull by rows: short rows only (central moments 128^3 81.9 -> 75.3 us, 192^3 266 -> 259, but
+  // 256^3 607 -> 628, 384^3 2109 -> 2164)
+  if (beyond_l2<S>(g) && (sizeof(S) == 2 || MODE != MODE_PULL || g.nx < 256))
     prefetch_ahead<S>(src, g, (uint64_t)(blockIdx.z + g.zb) * g.nxy +
                                   (uint64_t)blockIdx.y * g.nx + blockIdx.x * (2 * blockDim.x));
   const bool vb = xa + 32 < g.nx;
