@@ -72,11 +72,6 @@ VARIANTS = [
      "nu": 2e-4, "seed": 1, "storage": "f32", "scheme": "pull", "diag_every": 50, "steps": 100,
      "gamma": "exact", "gap": True},
 ]
-# FP64-pipe instructions per lattice update of step_kernel<double> (ncu: the FP64 pipe was
-# 86.8 % busy over 2.19 ms for 2,097,152 nodes, 571 instructions per node, on a 128^3 FP64
-# pull box) and the GB300 FP64 pipe peak of 2 instructions per SM per cycle.
-FP64_INSTR_PER_LUP = 571.0
-FP64_PIPE_PER_SM_PER_CYCLE = 2.0
 # DRAM bytes per lattice update of the default FP32 pull step kernel (packed FP32x2) from an ncu
 # capture, keyed by a hash of the kernel sources; a changed kernel gets no traffic figure until
 # it is profiled again.
@@ -111,7 +106,7 @@ def parse_workload(name):
     return w
 
 
-KERNEL_SOURCES = ("kbc_device.cuh", "kbc_kernels.cuh", "kbc_staged.cuh", "kbc_tma.cuh",
+KERNEL_SOURCES = ("kbc_device.cuh", "kbc_fix.cuh", "kbc_kernels.cuh", "kbc_staged.cuh", "kbc_tma.cuh",
                   "kbc_ops.h", "kbc_f32.cu", "kbc_f16.cu", "lb_api.cu")
 
 
@@ -298,8 +293,11 @@ def run_box(w, steps, warmup, want_kernel_time=True):
     total_ms = e_start.elapsed_time(e_end)
     step_ms = sum(a.elapsed_time(b) for a, b in ev)
     # per step the step kernel, plus the FP64 re-collision pass after it with FP32 storage
-    # (estimate of gamma); per diagnostics call two field kernels and two final sums
-    per_step = 2 if (w["storage"] == "f32" and w.get("gamma", "estimate") == "estimate") else 1
+    # (estimate of gamma), which even boxes of up to 2^18 nodes do in the step kernel; per
+    # diagnostics call two field kernels and two final sums
+    small = w["n"] ** 3 <= 2 ** 18 and w["n"] % 2 == 0
+    per_step = 2 if (w["storage"] == "f32" and w.get("gamma", "estimate") == "estimate"
+                     and not small) else 1
     launches = steps * per_step + 4 * len(diags)
     out = {"P": lat.P, "steps": steps, "total_ms": total_ms, "step_kernel_ms": step_ms / steps,
            "launches": launches, "diag": diags[-1] if diags else None, "lat": lat}
@@ -547,7 +545,7 @@ def main_ours(args, rank, world, local):
     rl = roofline(w["storage"], kernel_mlups, peak, peak_kind,
                   None if traffic is None else traffic * res["P"])
     rl["kernel"] = "kbc::%s<%s, %s>" % (
-        "step_kernel" if w["storage"] == "f64" else
+        "fix_step_kernel" if w["storage"] == "f64" else
         ("adj_step_kernel" if w["n"] % 2 == 0 else "pair_step_kernel"),
         {"f64": "double", "f32": "float", "f16": "uint16 (half bits)"}[w["storage"]],
         "MODE_PULL" if w["scheme"] == "pull" else "MODE_AA_EVEN/ODD")
@@ -556,8 +554,6 @@ def main_ours(args, rank, world, local):
     torch.cuda.empty_cache()
 
     variants = {}
-    clk_mhz = clk.summary().get("sm_mhz")
-    sms = torch.cuda.get_device_properties(local).multi_processor_count
     if not args.no_variants:
         chosen = VARIANTS if args.variants is None else [
             parse_workload(name) for name in args.variants.split(",") if name]
@@ -589,13 +585,9 @@ def main_ours(args, rank, world, local):
                             k: gp[k] for k in ("mean_abs", "max_abs", "mean_estimate",
                                                "mean_exact", "unconverged", "skipped")}
                     if v.get("gamma") == "exact":
-                        variants[v["name"]]["bound"] = "alu (Newton iterations)"
+                        variants[v["name"]]["bound"] = "alu (root of eq:result1)"
                     elif v["storage"] == "f64":
-                        sm_mhz = clk_mhz or 2070.0
-                        pipe_peak = FP64_PIPE_PER_SM_PER_CYCLE * sms * sm_mhz * 1e6
-                        variants[v["name"]]["bound"] = "alu (FP64 pipe)"
-                        variants[v["name"]]["frac_fp64_pipe"] = round(
-                            kml * 1e6 * FP64_INSTR_PER_LUP / pipe_peak, 4)
+                        variants[v["name"]]["bound"] = "alu (integer pipe, instruction fetch)"
                     del r["lat"]
                 torch.cuda.empty_cache()
             except Exception as e:  # report, do not hide

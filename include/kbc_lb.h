@@ -60,8 +60,9 @@ enum {
 };
 /* Stabilizer: eq:result21 (the method), the fixed special cases named in Sec. KBC
  * (gamma = 2, LBGK; gamma = 1/beta, regularized LB), or LB_GAMMA_EXACT: per node the root
- * gamma* of the entropy condition eq:result1, by a damped Newton iteration started from
- * eq:result21 (at most 50 iterations in FP64, 20 in FP32; each step halved until every
+ * gamma* of the entropy condition eq:result1, by a series around eq:result21 where every
+ * population's change is below a quarter of its equilibrium, else by a damped Newton iteration
+ * started from eq:result21 (at most 50 iterations in FP64, 20 in FP32; each step halved until every
  * logarithm's argument stays positive; nodes where <dh|dh> falls under the guard keep
  * gamma = 2). LB_GAMMA_EXACT runs in the one-node-per-thread direct kernel only and is not
  * available to batches. */
@@ -223,7 +224,7 @@ lb_status lb_get_populations(lb_ctx *ctx, double *f, int on_device);
  * (eq:result21, or 2 / 1/beta in the LBGK / RLB modes; 2 where <dh|dh> fell under the guard;
  * FP32, caller-owned gamma[P], node order). With LB_F32 storage, a node whose FP32 <dh|dh>
  * fell under 1e-13 is collided again in FP64 from its inputs (a second kernel after each
- * step kernel) and takes that gamma and those populations; LB_F16 storage keeps the FP32
+ * step kernel; in boxes of up to 2^18 nodes the step kernel itself) and takes that gamma and those populations; LB_F16 storage keeps the FP32
  * collision there. LB_ERR_INVALID_ARG when no step has run since the state was set.
  * Synchronises. */
 lb_status lb_get_gamma(lb_ctx *ctx, float *gamma, int on_device);
@@ -241,8 +242,9 @@ lb_status lb_set_time(lb_ctx *ctx, int64_t t);
 
 /* Which step kernel runs. All kernels give bit-identical populations for a given storage
  * (the FP32 kernels of one node per thread run the FP32x2 collision with the node in both
- * lanes, so every FP32 kernel executes the same compiled arithmetic). FP64 storage runs the
- * direct kernel.
+ * lanes, so every FP32 kernel executes the same compiled arithmetic). FP64 storage runs one
+ * node per thread: the estimate with natural moments and the product form in fixed point, in
+ * node order in blocks of bx * by (lb_set_block), all else in the direct kernel.
  *   LB_KERNEL_ROWS        two adjacent nodes per thread on packed FP32x2 instructions; a
  *                         persistent grid walks tiles of whole rows (nx <= 256) or 256-node
  *                         row segments (nx a multiple of 256), whose 27 source rows the
