@@ -130,7 +130,7 @@ template <typename S> __host__ __device__ inline bool beyond_l2(const Geo& g) {
 
 // Two nodes per thread with packed FP32x2 arithmetic: a block of up to 128 threads covers
 // 2 x blockDim.x consecutive x nodes of one row, each warp 64 of them as (x, x + 32) pairs.
-template <typename S, int MODE, bool RECORD, bool CENTRAL, bool POLY = false>
+template <typename S, int MODE, bool RECORD, bool CENTRAL, bool POLY, bool AHEAD>
 __global__ void __launch_bounds__(128, 3) pair_step_kernel(const S* src, S* dst, Geo g,
                                                         CollideParams cp, float* gamma_out,
                                                         StepCounters* ctr) {
@@ -138,9 +138,7 @@ __global__ void __launch_bounds__(128, 3) pair_step_kernel(const S* src, S* dst,
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t xa = blockIdx.x * (2 * blockDim.x) + warp * 64 + lane;
   if (xa >= g.nx) return;
-  // FP32 pull by rows: short rows only (central moments 128^3 81.9 -> 75.3 us, 192^3 266 -> 259, but
-  // 256^3 607 -> 628, 384^3 2109 -> 2164)
-  if (beyond_l2<S>(g) && (sizeof(S) == 2 || MODE != MODE_PULL || g.nx < 256))
+  if constexpr (AHEAD)
     prefetch_ahead<S>(src, g, (uint64_t)(blockIdx.z + g.zb) * g.nxy +
                                   (uint64_t)blockIdx.y * g.nx + blockIdx.x * (2 * blockDim.x));
   const bool vb = xa + 32 < g.nx;
@@ -316,8 +314,17 @@ static cudaError_t launch_pair(const S* src, S* dst, const Geo& g, const Collide
                             ctr);
   }
   const dim3 grid(row_blocks, g.ny, g.ze - g.zb);
-  return launch_following(pair_step_kernel<S, MODE, RECORD, CENTRAL, POLY>, grid, 32 * warps, st,
-                          src, dst, g, cp, gamma_out, ctr);
+  auto run = [&](auto ahead) {
+    return launch_following(
+        pair_step_kernel<S, MODE, RECORD, CENTRAL, POLY, decltype(ahead)::value>, grid, 32 * warps,
+        st, src, dst, g, cp, gamma_out, ctr);
+  };
+  // FP32 pull: short rows only (central moments without -> with: 128^3 81.9 -> 75.3 us, 192^3
+  // 266 -> 259, but 256^3 607 -> 628, 384^3 2109 -> 2164), and without the code for it, which
+  // costs those 3 % even where it is not taken
+  if (beyond_l2<S>(g) && (sizeof(S) == 2 || MODE != MODE_PULL || g.nx < 256))
+    return run(std::true_type{});
+  return run(std::false_type{});
 }
 
 // the geometry and collision parameters of box `bd` of a batch (the whole box is stepped;
