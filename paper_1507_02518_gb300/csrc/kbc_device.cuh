@@ -55,12 +55,8 @@ template <> struct Codec<double> {
   using R = double;
   static constexpr bool rel = false;
   template <int I> __device__ static __forceinline__ R load(const double* p) { return *p; }
-  template <int I> __device__ static __forceinline__ R load_ro(const double* p) { return __ldg(p); }
   template <int I> __device__ static __forceinline__ void store(double* p, R d) { *p = d; }
   template <int I> __device__ static __forceinline__ R load_raw(const double* p) { return *p; }
-  template <int I> __device__ static __forceinline__ R load_raw_ro(const double* p) {
-    return __ldg(p);
-  }
   template <int I> __device__ static __forceinline__ void store_raw(double* p, R d) { *p = d; }
   __host__ __device__ static double to_delta(double s, int) { return s; }
   __host__ __device__ static double from_delta(double d, int) { return d; }
@@ -70,12 +66,8 @@ template <> struct Codec<float> {
   using R = float;
   static constexpr bool rel = false;
   template <int I> __device__ static __forceinline__ R load(const float* p) { return *p; }
-  template <int I> __device__ static __forceinline__ R load_ro(const float* p) { return __ldg(p); }
   template <int I> __device__ static __forceinline__ void store(float* p, R d) { *p = d; }
   template <int I> __device__ static __forceinline__ R load_raw(const float* p) { return *p; }
-  template <int I> __device__ static __forceinline__ R load_raw_ro(const float* p) {
-    return __ldg(p);
-  }
   template <int I> __device__ static __forceinline__ void store_raw(float* p, R d) { *p = d; }
   __device__ static double to_delta(float s, int) { return (double)s; }
   __device__ static float from_delta(double d, int) { return (float)d; }
@@ -89,17 +81,11 @@ template <> struct Codec<uint16_t> {
   template <int I> __device__ static __forceinline__ R load(const uint16_t* p) {
     return __fmul_rn((float)wgt(I), __half2float(__ushort_as_half(*p)));
   }
-  template <int I> __device__ static __forceinline__ R load_ro(const uint16_t* p) {
-    return __fmul_rn((float)wgt(I), __half2float(__ushort_as_half(__ldg(p))));
-  }
   template <int I> __device__ static __forceinline__ void store(uint16_t* p, R d) {
     *p = __half_as_ushort(__float2half_rn(__fmul_rn(d, (float)inv_wgt(I))));
   }
   template <int I> __device__ static __forceinline__ R load_raw(const uint16_t* p) {
     return __half2float(__ushort_as_half(*p));
-  }
-  template <int I> __device__ static __forceinline__ R load_raw_ro(const uint16_t* p) {
-    return __half2float(__ushort_as_half(__ldg(p)));
   }
   template <int I> __device__ static __forceinline__ void store_raw(uint16_t* p, R d) {
     *p = __half_as_ushort(__float2half_rn(d));
@@ -116,9 +102,9 @@ template <> struct Codec<uint16_t> {
 // store_raw above), for the packed kernels.
 template <typename S> struct Codec2;
 template <> struct Codec2<float> {
-  template <int I, bool RO>
+  template <int I>
   __device__ static __forceinline__ float2 load(const float* pa, const float* pb) {
-    return RO ? make_float2(__ldg(pa), __ldg(pb)) : make_float2(*pa, *pb);
+    return make_float2(*pa, *pb);
   }
   template <int I> __device__ static __forceinline__ void store(float* pa, float* pb, bool va,
                                                               bool vb, float2 v) {
@@ -127,10 +113,9 @@ template <> struct Codec2<float> {
   }
 };
 template <> struct Codec2<uint16_t> {
-  template <int I, bool RO>
+  template <int I>
   __device__ static __forceinline__ float2 load(const uint16_t* pa, const uint16_t* pb) {
-    const uint16_t a = RO ? __ldg(pa) : *pa, b = RO ? __ldg(pb) : *pb;
-    return __half22float2(__halves2half2(__ushort_as_half(a), __ushort_as_half(b)));
+    return __half22float2(__halves2half2(__ushort_as_half(*pa), __ushort_as_half(*pb)));
   }
   template <int I> __device__ static __forceinline__ void store(uint16_t* pa, uint16_t* pb,
                                                               bool va, bool vb, float2 v) {
@@ -144,27 +129,23 @@ template <> struct Codec2<uint16_t> {
 // give a thread two neighbouring nodes of a row: v0, vl and vr point at the values of nodes x,
 // x - 1 and x + 2 (row neighbours, periodic wrap already applied); SX selects the pair read,
 // nodes (x + SX, x + 1 + SX). The unshifted pair is one 32-bit (FP16) or 64-bit (FP32) access
-// (x even, rows of even length); a shifted pair is two scalar accesses. RO: read-only path.
+// (x even, rows of even length); a shifted pair is two scalar accesses.
 template <typename S> struct PairIO;
 template <> struct PairIO<uint16_t> {
-  template <bool RO> __device__ static __forceinline__ uint16_t ld1(const uint16_t* p) {
-    return RO ? __ldg(p) : *p;
-  }
-  template <int SX, bool RO>
+  template <int SX>
   __device__ static __forceinline__ float2 get(const uint16_t* v0, const uint16_t* vl,
                                                const uint16_t* vr) {
     if constexpr (SX == 0) {
-      const unsigned int w = RO ? __ldg(reinterpret_cast<const unsigned int*>(v0))
-                                : *reinterpret_cast<const unsigned int*>(v0);
+      const unsigned int w = *reinterpret_cast<const unsigned int*>(v0);
       __half2 h;
       memcpy(&h, &w, sizeof h);
       return __half22float2(h);
     } else if constexpr (SX < 0) {
       return __half22float2(
-          __halves2half2(__ushort_as_half(ld1<RO>(vl)), __ushort_as_half(ld1<RO>(v0))));
+          __halves2half2(__ushort_as_half(*vl), __ushort_as_half(*v0)));
     } else {
       return __half22float2(
-          __halves2half2(__ushort_as_half(ld1<RO>(v0 + 1)), __ushort_as_half(ld1<RO>(vr))));
+          __halves2half2(__ushort_as_half(v0[1]), __ushort_as_half(*vr)));
     }
   }
   __device__ static __forceinline__ void put2(uint16_t* p, float2 v) {
@@ -175,19 +156,15 @@ template <> struct PairIO<uint16_t> {
   }
 };
 template <> struct PairIO<float> {
-  template <bool RO> __device__ static __forceinline__ float ld1(const float* p) {
-    return RO ? __ldg(p) : *p;
-  }
-  template <int SX, bool RO>
+  template <int SX>
   __device__ static __forceinline__ float2 get(const float* v0, const float* vl,
                                                const float* vr) {
     if constexpr (SX == 0) {
-      return RO ? __ldg(reinterpret_cast<const float2*>(v0))
-                : *reinterpret_cast<const float2*>(v0);
+      return *reinterpret_cast<const float2*>(v0);
     } else if constexpr (SX < 0) {
-      return make_float2(ld1<RO>(vl), ld1<RO>(v0));
+      return make_float2(*vl, *v0);
     } else {
-      return make_float2(ld1<RO>(v0 + 1), ld1<RO>(vr));
+      return make_float2(v0[1], *vr);
     }
   }
   __device__ static __forceinline__ void put2(float* p, float2 v) {
@@ -1439,8 +1416,7 @@ __device__ __forceinline__ float fix_node_update(const S* src, S* dst, const Geo
   S d[27];
   Unroll<0, 27>::run([&](auto ic) {
     constexpr int I = decltype(ic)::value;
-    const S* p = src + (uint64_t)Pat::load_plane(I) * g.P + nb.template at<I, Pat::load_shift>();
-    d[I] = MODE == MODE_PULL ? __ldg(p) : *p;
+    d[I] = src[(uint64_t)Pat::load_plane(I) * g.P + nb.template at<I, Pat::load_shift>()];
   });
   fix::fx v[27];
   double gam;
@@ -1480,11 +1456,7 @@ __device__ __forceinline__ void node_update(const S* src, S* dst, const Geo& g, 
   Unroll<0, 27>::run([&](auto ic) {
     constexpr int I = decltype(ic)::value;
     const S* p = src + (uint64_t)Pat::load_plane(I) * g.P + nb.template at<I, Pat::load_shift>();
-    if constexpr (MODE == MODE_PULL) {
-      d[I] = C::template load_raw_ro<I>(p);
-    } else {
-      d[I] = C::template load_raw<I>(p);
-    }
+    d[I] = C::template load_raw<I>(p);
   });
   int guarded, fp64 = 0;
   R gamma = collide_step<R, CENTRAL, EXACT, POLY, C::rel>(
@@ -1530,7 +1502,7 @@ __device__ __forceinline__ void node_update2(const S* src, S* dst, const Geo& g,
   Unroll<0, 27>::run([&](auto ic) {
     constexpr int I = decltype(ic)::value;
     const S* base = src + (uint64_t)Pat::load_plane(I) * g.P;
-    d[I] = Codec2<S>::template load<I, MODE == MODE_PULL>(
+    d[I] = Codec2<S>::template load<I>(
         base + na.template at<I, Pat::load_shift>(), base + nb.template at<I, Pat::load_shift>());
   });
   int guarded, fp64 = 0;
@@ -1624,7 +1596,7 @@ __device__ __forceinline__ void node_update_adj(const S* src, S* dst, const Geo&
     constexpr int LS = Pat::load_shift;
     const S* plane = src + (uint64_t)Pat::load_plane(I) * g.P;
     const uint32_t o1 = oy[LS * cy(I) + 1], o2 = oz[LS * cz(I) + 1];
-    d[I] = IO::template get<LS * cx(I), MODE == MODE_PULL>(
+    d[I] = IO::template get<LS * cx(I)>(
         at(plane, o1, o2, x), at(plane, o1, o2, xm), at(plane, o1, o2, xp2));
   });
   int guarded, fp64 = 0;

@@ -33,6 +33,9 @@ template <> struct MaxThreads<double> { static constexpr int value = 256; };
 // adjacent-pair steps let the next kernel in at their end only (let_next(): 32^3 FP32 pull 3.9 ->
 // 3.4 us, AA without a pass 4.6 -> 3.2), and the FP64 step, whose blocks fill an SM with three, when
 // its blocks exit (32^3 11.2 -> 8.7 us).
+// Populations are read by ordinary loads only: __ldg() and ld.global.nc are for memory that nothing
+// writes while the kernel lives, and a kernel of the chain lives while the one before writes what
+// it will read (with small grids also while the one before that still reads the same buffer).
 __device__ __forceinline__ void wait_before() { cudaGridDependencySynchronize(); }
 __device__ __forceinline__ void let_next() { cudaTriggerProgrammaticLaunchCompletion(); }
 __device__ __forceinline__ void follow() {

@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(kRowsThreads, 3)
       Unroll<0, 27>::run([&](auto ic) {
         constexpr int I = decltype(ic)::value;
         constexpr int SX = Pat::load_shift * cx(I);
-        d[I] = LD::template get<SX, false>(v0 + I * L::PS, vl + I * L::PS, vr + I * L::PS);
+        d[I] = LD::template get<SX>(v0 + I * L::PS, vl + I * L::PS, vr + I * L::PS);
       });
     }
     __syncwarp();
