@@ -1211,23 +1211,24 @@ template <int N> struct Unroll<N, N> {
 };
 
 // The fixed-point collision (kbc_fix.cuh) of the shifts d (FP64 or FP32 values), the result in
-// v (to_f64<nonzero(i)>). False when the node is outside the format's range: v is then nothing,
-// and the caller collides in FP64.
-template <typename S>
-__device__ __forceinline__ bool fix_collide(const S (&d)[27], fix::fx (&v)[27],
+// v (to_f64<nonzero(i)>, scale *s; CHANGE: f' - f). False when the node is outside the format's
+// range: v is then nothing, and the caller collides in FP64.
+template <bool CHANGE, typename S>
+__device__ __forceinline__ bool fix_collide(const S (&d)[27], fix::fx (&v)[27], uint32_t* s,
                                             const CollideParams& cp, int* guarded,
                                             double* gamma) {
   uint32_t top = 0;
 #pragma unroll
-  for (int i = 0; i < 27; ++i) {
-    if constexpr (std::is_same<S, double>::value) v[i] = fix::from_f64(d[i], &top);
-    else v[i] = fix::from_f32(d[i], &top);
-  }
-  if (top >= (std::is_same<S, double>::value ? fix::kTopF64 : fix::kTopF32)) return false;
+  for (int i = 0; i < 27; ++i) top = fix::top_of(d[i]) > top ? fix::top_of(d[i]) : top;
+  if (top >= (std::is_same<S, double>::value ? fix::kTopF64 : fix::kTopF32) ||
+      !fix::scale_of<S>(top, s))
+    return false;
+#pragma unroll
+  for (int i = 0; i < 27; ++i) v[i] = fix::scaled(d[i], *s);
   const fix::Relax rx = {cp.quarter_beta, cp.two_beta_1, cp.inv_beta,
                          cp.with_t,       cp.with_q,     cp.gamma_mode};
   bool bad;
-  *gamma = fix::collide(v, rx, guarded, &bad);
+  *gamma = fix::collide<CHANGE>(v, rx, guarded, &bad, *s);
   return !bad;
 }
 
@@ -1259,13 +1260,15 @@ __device__ __forceinline__ R collide_step(R (&d)[27], const CollideParams& cp, i
       return collide_lean<R, REL>(d, cp, guarded, fp64);
     }
   } else if constexpr (!CENTRAL && !EXACT && !POLY) {
-    // FP64: the fixed-point collision, or this one in FP64 where the node is outside its range
+    // FP64: the fixed-point collision as fix_node_update() adds it, or this one in FP64 where the
+    // node is outside its range
     fix::fx v[27];
     double gam;
-    if (fix_collide(d, v, cp, guarded, &gam)) {
+    uint32_t s;
+    if (fix_collide<true>(d, v, &s, cp, guarded, &gam)) {
       Unroll<0, 27>::run([&](auto ic) {
         constexpr int I = decltype(ic)::value;
-        d[I] = fix::to_f64<fix::nonzero(I)>(v[I]);
+        d[I] = __dadd_rn(d[I], fix::to_f64<fix::nonzero(I)>(v[I], s));
       });
       return gam;
     }
@@ -1405,27 +1408,54 @@ __device__ __noinline__ float fp64_node_native(const S* src, S* dst, Geo g, uint
 // The FP64 update of one node (FP64 storage: every step; FP32 storage: the re-collision of a
 // node whose FP32 <dh|dh> fell under kDenFp64) with the fixed-point collision, natural moments
 // and product form. Returns gamma; *guarded is set when <dh|dh> vanished.
+//
+// FP64 storage adds the change f' - f to the stored shift in FP64: the collision takes the shifts to
+// a grid of 2^-55 of the node's largest, and what a shift has below that stays with it this way.
+// The conserved moments of the change are exactly 0, so that mass and momentum drift by the
+// rounding of one addition per population only. (Without it the residues of a uniform flow, which are
+// the same every step, add up.) The populations are read again for that, from the first level of
+// the cache: held across the collision they would take 54 registers.
 template <typename S, int MODE>
 __device__ __forceinline__ float fix_node_update(const S* src, S* dst, const Geo& g, uint32_t x,
                                                  uint32_t y, uint32_t z,
                                                  const CollideParams& cp, int* guarded) {
   using C = Codec<S>;
   using Pat = Pattern<MODE>;
-  Nbr nb;
-  nb.init(g, x, y, z);
+  constexpr bool CHANGE = std::is_same<S, double>::value;
   S d[27];
-  Unroll<0, 27>::run([&](auto ic) {
-    constexpr int I = decltype(ic)::value;
-    d[I] = src[(uint64_t)Pat::load_plane(I) * g.P + nb.template at<I, Pat::load_shift>()];
-  });
+  {
+    Nbr nb;
+    nb.init(g, x, y, z);
+    Unroll<0, 27>::run([&](auto ic) {
+      constexpr int I = decltype(ic)::value;
+      d[I] = src[(uint64_t)Pat::load_plane(I) * g.P + nb.template at<I, Pat::load_shift>()];
+    });
+  }
   fix::fx v[27];
   double gam;
-  if (!fix_collide(d, v, cp, guarded, &gam))
+  uint32_t s;
+  if (!fix_collide<CHANGE>(d, v, &s, cp, guarded, &gam))
     return fp64_node_native<S, MODE, false, false>(src, dst, g, x, y, z, cp, guarded);
+  // from coordinates that the compiler takes for new ones: the neighbour offsets are then not kept
+  // across the collision
+  asm volatile("" : "+r"(x), "+r"(y), "+r"(z));
+  Nbr nb;
+  nb.init(g, x, y, z);
+  if constexpr (CHANGE) {
+    Unroll<0, 27>::run([&](auto ic) {
+      constexpr int I = decltype(ic)::value;
+      asm volatile("ld.global.f64 %0, [%1];"
+                   : "=d"(d[I])
+                   : "l"(src + (uint64_t)Pat::load_plane(I) * g.P +
+                         nb.template at<I, Pat::load_shift>())
+                   : "memory");
+    });
+  }
   Unroll<0, 27>::run([&](auto ic) {
     constexpr int I = decltype(ic)::value;
+    const double r = fix::to_f64<fix::nonzero(I)>(v[I], s);
     dst[(uint64_t)Pat::store_plane(I) * g.P + nb.template at<I, Pat::store_shift>()] =
-        C::from_delta(fix::to_f64<fix::nonzero(I)>(v[I]), I);
+        CHANGE ? __dadd_rn(d[I], r) : C::from_delta(r, I);
   });
   return (float)gam;
 }

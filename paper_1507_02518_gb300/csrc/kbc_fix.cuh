@@ -4,10 +4,16 @@
 // integer additions, shifts and logic operations (a 64-bit addition of two or three terms is
 // two instructions) and 64 32-bit multiplies (measured). An FP64 collision in FP64 instructions
 // (571 of them per node) is bound by that pipe at 6 % of the memory roof. Here the shifts f - W,
-// their moments and the equilibrium are integers of unit 2^-60 instead: |f - W| < 1/4 then has at
-// least the resolution that f itself has in FP64 (f >= 2^-8), sums are exact, products are good
-// to two units, and the absolute error of the result is ~2e-18 where FP64 arithmetic leaves
-// ~2.5e-17 (its sqrt(1 + 3u^2) alone is rounded at 2^-53).
+// their moments and the equilibrium are integers instead, of a unit that follows the node: its
+// largest shift has 55 bits (a unit of 2^-60 for shifts above 2^-6), so that nothing is lost at
+// small amplitudes either. Sums are exact, products good to 3/4 of a unit. FP64 storage adds the
+// change f' - f, whose conserved moments are exactly 0, to the stored shift: what a shift has below
+// the unit stays with it, and mass and momentum drift by the rounding of that addition only.
+// Against extended precision, relative to the node's largest shift, rms over nodes of amplitudes
+// 0.12 to 1e-17: 4e-17..7e-17, FP64 instructions 1.0e-16..1.5e-16; 10^4 collisions of a uniform flow
+// change its mass and momentum by 5e-16..1.1e-14 of it, FP64 instructions by 1e-15..2.6e-13. gamma
+// is good to 4e-16..7e-16 far from equilibrium (FP64 2e-16..3e-16) and to less than FP64's error
+// nearer to it.
 //   * everything linear in f (moments, deviations, relaxation, back transform) is done on the
 //     27 natural moments with integer additions; the relaxation multiplies 23 moments, not
 //     2 x 27 populations;
@@ -15,15 +21,15 @@
 //     corrected by Newton's method with integer residuals;
 //   * the entropic products, of which a ratio is taken, are integer products too, of deviations
 //     scaled by a common power of two to about 2^59, with integer weights that need no
-//     reciprocal; their sums are good to about 2^-47.
-// About 3400 instructions per node, of which 27 (the conversions of the results) are the FP64
-// pipe's; what bounds it is the integer pipe (54 % busy) and instruction fetch at 12 warps per SM.
-// Measured at 256^3 (FP64 pull): FP64 instructions 17.4 ms a step, this with the entropic
-// products in FP32 pairs (two-sum, two-product) 4.4 ms, in integers 2.8 ms; 432 B a node take
-// 1.08 ms. Taking the inputs' conversions to the FP64 pipe, or the results' by two additions
-// there, changed nothing (2.80, 3.42 against 2.83, 3.43 ms).
-// Nodes outside the range of the format (|f - W| >= 1/4, rho or u far from a lattice state,
-// NaN, |beta gamma| >= 128) are reported and left to the FP64 collision.
+//     reciprocal.
+// About 3500 instructions per node, of which 54 (the conversions of the changes and the additions)
+// are the FP64 pipe's, which they fill for nearly half of the time; 16 warps per SM.
+// Measured at 256^3 (FP64 pull): FP64 instructions 17.4 ms a step, this 3.2 ms; 432 B a node take
+// 1.08 ms. A fixed unit of 2^-60, without the change and with products rounded down took 2.85 ms (32^3
+// 8.7 us, now 11.3) but lost momentum one-sidedly, and small shifts their bits. The sum in integers
+// instead of FP64: 3.48 ms.
+// Nodes outside the range of the format (|f - W| >= 1/4 or all below 2^-70, rho or u far from a
+// lattice state, NaN, |beta gamma| >= 128) are reported and left to the FP64 collision.
 //
 // The functions are host code as well (no CUDA intrinsics there), so that they can be checked
 // without a GPU.
@@ -92,6 +98,24 @@ KBC_HD uint64_t shr(uint64_t x, uint32_t n) {
   return n > 63 ? 0 : x >> n;
 #endif
 }
+KBC_HD fx sar(fx x, uint32_t n) {
+#ifdef __CUDA_ARCH__
+  fx r;
+  asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(n));
+  return r;
+#else
+  return x >> (n > 63 ? 63 : n);
+#endif
+}
+KBC_HD int32_t sar32(int32_t x, uint32_t n) {
+#ifdef __CUDA_ARCH__
+  int32_t r;
+  asm("shr.s32 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(n));
+  return r;
+#else
+  return x >> (n > 31 ? 31 : n);
+#endif
+}
 KBC_HD float rcpf(float x) {
 #ifdef __CUDA_ARCH__
   float r;
@@ -141,29 +165,57 @@ KBC_HD int clz64(uint64_t x) {
 #endif
 }
 
-// d as a fixed-point number, truncated; *top collects the largest high word of |d|, by which
-// the caller sees values (and NaN) outside the range
-KBC_HD fx from_f64(double d, uint32_t* top) {
-  const uint64_t b = bits_of(d);
-  const uint32_t hi = (uint32_t)(b >> 32), ah = hi & 0x7fffffffu;
-  *top = ah > *top ? ah : *top;
-  const uint64_t m = (b << 11) | 0x8000000000000000ull;  // 1.mantissa, leading bit at 63
-  const fx x = (fx)shr(m, 1026u - (ah >> 20));           // 0 for |d| < 2^-61, zero included
-  return (int32_t)hi < 0 ? -x : x;
+// The high word of |d| (FP32: |d|); its largest over a node tells the caller whether the values
+// (NaN among them) are in the range, and the node's scale.
+KBC_HD uint32_t top_of(double d) { return (uint32_t)(bits_of(d) >> 32) & 0x7fffffffu; }
+KBC_HD uint32_t top_of(float d) { return bits_of(d) & 0x7fffffffu; }
+
+// A node's scale s: its numbers are integers of unit 2^-(60 + s), so that small shifts keep their
+// bits. s puts the largest shift into [1/2, 1) 2^-5 (the room to 1/4 is for the moments, sums of
+// many shifts), and is 0 where it is larger than that. False for shifts that are all below
+// 2^-6 2^-kMaxScale but not zero.
+constexpr uint32_t kMaxScale = 64;
+template <typename T, uint32_t EXP> KBC_HD bool scale_to(uint32_t top, uint32_t* s) {
+  const uint32_t bias = sizeof(T) == 8 ? 1023 : 127, e = top >> (sizeof(T) == 8 ? 20 : 23);
+  const uint32_t want = bias - EXP - 1;  // biased exponent of the values in [1/2, 1) 2^-EXP
+  *s = e < want && top != 0 ? want - e : 0;
+  return *s <= kMaxScale;
 }
-KBC_HD fx from_f32(float d, uint32_t* top) {
-  const uint32_t b = bits_of(d), ah = b & 0x7fffffffu;
-  *top = ah > *top ? ah : *top;
+template <typename T> KBC_HD bool scale_of(uint32_t top, uint32_t* s) {
+  return scale_to<T, 5>(top, s);
+}
+
+// d 2^s as a fixed-point number, truncated
+KBC_HD fx scaled(double d, uint32_t s) {
+  const uint64_t b = bits_of(d);
+  const uint64_t m = (b << 11) | 0x8000000000000000ull;  // 1.mantissa, leading bit at 63
+  // 0 for |d| < 2^-61, zero included
+  const fx x = (fx)shr(m, 1026u - s - ((uint32_t)(b >> 52) & 0x7ffu));
+  return (int64_t)b < 0 ? -x : x;
+}
+KBC_HD fx scaled(float d, uint32_t s) {
+  const uint32_t b = bits_of(d);
   const uint64_t m = (uint64_t)((b << 8) | 0x80000000u) << 32;
-  const fx x = (fx)shr(m, 130u - (ah >> 23));
+  const fx x = (fx)shr(m, 130u - s - ((b >> 23) & 0xffu));
   return (int32_t)b < 0 ? -x : x;
 }
-// v * 2^-(60 + n), rounded to nearest even: one conversion and an exponent shift (|v| < 2^63;
+// the same for s = 0; *top collects the largest top_of()
+KBC_HD fx from_f64(double d, uint32_t* top) {
+  const uint32_t ah = top_of(d);
+  *top = ah > *top ? ah : *top;
+  return scaled(d, 0);
+}
+KBC_HD fx from_f32(float d, uint32_t* top) {
+  const uint32_t ah = top_of(d);
+  *top = ah > *top ? ah : *top;
+  return scaled(d, 0);
+}
+// v * 2^-(60 + n + s), rounded to nearest even: one conversion and an exponent shift (|v| < 2^63;
 // the result is normal or zero)
-template <int N> KBC_HD double to_f64(fx v) {
+template <int N> KBC_HD double to_f64(fx v, uint32_t s = 0) {
   const uint64_t b = bits_of((double)v);
   uint32_t hi = (uint32_t)(b >> 32);
-  hi = hi == 0 ? 0 : hi - ((uint32_t)(kFrac + N) << 20);
+  hi = hi == 0 ? 0 : hi - ((kFrac + N + s) << 20);
   return f64_of((uint64_t)hi << 32 | (uint32_t)b);
 }
 
@@ -240,25 +292,35 @@ KBC_HD constexpr int32_t mul_high(int32_t a, int32_t b) {
   return (int32_t)(((long long)a * b) >> 32);
 #endif
 }
-// a b / 2^64 with both cross terms rounded down and l x l (less than 1/4 unit) dropped: one
-// 32 x 32 -> 64 bit multiply and two high halves, 4 instructions; 0 to 2 1/4 units below the
-// product (none for a factor 0). |a| < 2^62.9 and |b| < 2^63 - 2^31 keep the cross terms' sum in
-// 32 bits.
-KBC_HD constexpr fx mul(Split a, Split b) {
+// a b / 2^64 to nearest, but for l x l (less than 1/4 unit, of either sign), which is dropped:
+// within 3/4 of a unit, 0 for a factor 0. |a| < 2^62.9 and |b| < 2^63 - 2^31 keep the cross terms'
+// sum in 64 bits.
+KBC_HD fx mul(Split a, Split b) {
+#ifdef __CUDA_ARCH__
+  long long c, r;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(c) : "r"(a.l), "r"(b.h), "l"(0x80000000ll));
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(c) : "r"(a.h), "r"(b.l), "l"(c));
+  asm("mad.wide.s32 %0, %1, %2, %3;"
+      : "=l"(r)
+      : "r"(a.h), "r"(b.h), "l"((long long)(int32_t)(c >> 32)));
+  return r;
+#else
+  const long long c = (long long)a.h * b.l + ((long long)a.l * b.h + 0x80000000ll);
+  return (long long)a.h * b.h + (int32_t)(c >> 32);
+#endif
+}
+// The same with each cross term rounded down, a unit low on average unless a factor is 0: two high
+// halves instead of two wide multiplies, which take twice as long (256^3 FP64 pull with every product
+// to nearest 3.45 ms, with the 81 innermost entropic ones by this 3.2). For sums that start with
+// what they will lose.
+KBC_HD fx mul_down(Split a, Split b) {
   return (long long)a.h * b.h + (mul_high(a.h, b.l) + mul_high(a.l, b.h));
 }
 // a factor below 1/2 in magnitude, scaled by 2^4 so that mul() gives a product of unit 2^-60
 KBC_HD constexpr Split factor(fx v) { return split((fx)((uint64_t)v << 4)); }
 
-// 1/3 (rounded), and 1/9 and 1/27 as mul() gives them, so that the deviations of a node at
-// rest are exactly 0
+// 1/3 (rounded)
 constexpr fx kThird = 384307168202282325ll;
-KBC_HD constexpr long long high_of(long long a, long long b) { return (a * b) >> 32; }
-KBC_HD constexpr fx mul_const(Split a, Split b) {
-  return (long long)a.h * b.h + (int32_t)(high_of(a.h, b.l) + high_of(a.l, b.h));
-}
-constexpr fx kNinth = mul_const(split(kThird), factor(kThird));
-constexpr fx k27th = mul_const(split(kNinth), factor(kThird));
 
 // 1 / rho for 0.4 < rho < 2: FP32 reciprocal r0 in units of 2^-28, then r0 (1 + E + E^2) with
 // E = 1 - rho r0 to 2^-58 (|E| < 2^-21, so E^3 < 2^-63)
@@ -273,27 +335,31 @@ KBC_HD fx reciprocal(fx rho) {
   return ((fx)r0 << 32) + (((long long)r0 * Eh) >> 12) + mul_high(r0, El << 4);
 }
 
-// e = sqrt(1 + 3u^2) - 1, the root of e^2 + 2e = t = 3u^2, for |u| < 1/4 (e < 0.09): an FP32
-// value e0 (unit 2^-32, good to 2^-24), then x = d - g d^2 with d = g r, r = t - 2 e0 - e0^2 exact
-// in integers and g = 1 / (2 + 2 e0) to 2^-30 (one Newton step on the FP32 reciprocal)
-KBC_HD fx axis_e(Split u4, fx u) {
-  const fx uu = mul(split(u), u4);
+// e 2^s with e = sqrt(1 + 3u^2) - 1, the root of e^2 + 2e = t = 3u^2, for |u| 2^s < 1/4 (us is
+// u 2^s, u4 the factor of u; ps = 2^-s): an FP32 value e0 of e 2^s (unit 2^-32, good to 2^-24), then
+// x = d - g d^2 2^-s with d = g r, r = t 2^s - 2 e0 - e0^2 2^-s exact in integers and
+// g = 1 / (2 + 2e) to 2^-30 (one Newton step on the FP32 reciprocal)
+KBC_HD fx axis_e(Split u4, fx us, uint32_t s, float ps) {
+  const fx uu = mul(split(us), u4);
   const fx t = uu + uu + uu;
   const float tf = mulf((float)(int32_t)(t >> 29), 1.0f / 2147483648.0f);
-  const float ef = mulf(tf, rcpf(addf(1.0f, sqrtf_fast(addf(1.0f, tf)))));
+  const float ef = mulf(tf, rcpf(addf(1.0f, sqrtf_fast(addf(1.0f, mulf(tf, ps))))));
   const int32_t e0 = f2i(mulf(ef, 4294967296.0f));
-  const fx r = t - ((fx)e0 << 29) - (((long long)e0 * e0) >> 4);  // |r| < 2^37
-  int32_t g = f2i(mulf(rcpf(addf(1.0f, ef)), 1073741824.0f));     // 1 / (1 + e0) of 2^30
-  // g (1 + e0) of 2^60, less 1, over 2^30
-  const int32_t off = (int32_t)((((long long)g << 30) + (((long long)g * e0) >> 2) - kOne) >> 30);
+  const fx r = t - ((fx)e0 << 29) - sar(((long long)e0 * e0) >> 4, s);  // |r| < 2^37
+  int32_t g = f2i(mulf(rcpf(addf(1.0f, mulf(ef, ps))), 1073741824.0f));  // 1 / (1 + e) of 2^30
+  // g (1 + e) of 2^60, less 1, over 2^30
+  const int32_t off =
+      (int32_t)((((long long)g << 30) + sar(((long long)g * e0) >> 2, s) - kOne) >> 30);
   g -= off;
-  // r / (2 (1 + e0)) of 2^63
+  // r / (2 (1 + e)) of 2^63
   const long long d =
       ((long long)(int32_t)(r >> 6) * g + (mul_high((int32_t)(r & 63) << 25, g) << 1)) >> 22;
   const int32_t ds = (int32_t)(d >> 9);                 // of 2^54, below 2^31
-  const int32_t x2 = mul_high(mul_high(ds, ds), g);     // d^2 / (1 + e0) of 2^74
-  return ((fx)e0 << 28) + ((d - (x2 >> 12)) >> 3);
+  const int32_t x2 = mul_high(mul_high(ds, ds), g);     // d^2 / (1 + e) of 2^74
+  return ((fx)e0 << 28) + ((d - sar32(x2, s + 12)) >> 3);
 }
+// 2^-s
+KBC_HD float pow2_of(uint32_t s) { return f32_of((127 - s) << 23); }
 
 // ------------------------------------------------------------------ transforms
 // natural moments M[p + 3q + 9r] = sum_i f_i vx^p vy^q vz^r (eq:natmoments), in place: per axis
@@ -344,22 +410,25 @@ KBC_HD int clz32(uint32_t x) {
 }
 KBC_HD fx shl(fx v, int n) { return (fx)((uint64_t)v << n); }
 
-// f_eq(1 + drho, u) - W for |drho| < 1/4, |u_a| < 1/4: its moments, transformed back; population
-// i times 2^nonzero(i)
-KBC_HD void equilibrium(fx drho, fx ux, fx uy, fx uz, fx (&m)[27]) {
-  const Split ux4 = factor(ux), uy4 = factor(uy), uz4 = factor(uz);
+// f_eq(1 + drho, u) - W, times 2^s, for drho 2^s and u 2^s below 1/4: its moments, transformed
+// back; population i times 2^nonzero(i). The sum of the populations is drho exactly. The moments are
+// built from what they deviate by from those of the weights, which scales like the shifts:
+// rho m_2 - 1/3 = drho m_2 + (m_2 - 1/3), and so on.
+KBC_HD void equilibrium(fx drho, fx ux, fx uy, fx uz, fx (&m)[27], uint32_t s = 0) {
+  const float ps = pow2_of(s);
+  const Split ux4 = factor(sar(ux, s)), uy4 = factor(sar(uy, s)), uz4 = factor(sar(uz, s));
   const Split third = factor(kThird);
-  const fx ex = axis_e(ux4, ux), ey = axis_e(uy4, uy), ez = axis_e(uz4, uz);
-  const Split wx4 = factor(kThird + mul(split(ex + ex), third));
-  const Split wy4 = factor(kThird + mul(split(ey + ey), third));
-  const Split wz4 = factor(kThird + mul(split(ez + ez), third));
-  const Split rs = split(kOne + drho);
-  const fx rwx = mul(rs, wx4), rwy = mul(rs, wy4);
-  const Split rwxs = split(rwx);
+  const fx ex = axis_e(ux4, ux, s, ps), ey = axis_e(uy4, uy, s, ps), ez = axis_e(uz4, uz, s, ps);
+  // second moments of the axis factors less 1/3: 2e/3
+  const fx vx = mul(split(ex + ex), third), vy = mul(split(ey + ey), third),
+           vz = mul(split(ez + ez), third);
+  const Split wx4 = factor(kThird + sar(vx, s)), wy4 = factor(kThird + sar(vy, s)),
+              wz4 = factor(kThird + sar(vz, s));
+  const Split rs = split(drho);
   m[mi(0, 0, 0)] = drho;
-  m[mi(1, 0, 0)] = mul(rs, ux4);
-  m[mi(0, 1, 0)] = mul(rs, uy4);
-  m[mi(0, 0, 1)] = mul(rs, uz4);
+  m[mi(1, 0, 0)] = ux + mul(rs, ux4);
+  m[mi(0, 1, 0)] = uy + mul(rs, uy4);
+  m[mi(0, 0, 1)] = uz + mul(rs, uz4);
   const Split jxs = split(m[mi(1, 0, 0)]), jys = split(m[mi(0, 1, 0)]);
   const Split jzs = split(m[mi(0, 0, 1)]);
   m[mi(1, 1, 0)] = mul(jxs, uy4);
@@ -379,14 +448,15 @@ KBC_HD void equilibrium(fx drho, fx ux, fx uy, fx uz, fx (&m)[27]) {
   m[mi(2, 2, 1)] = mul(split(m[mi(2, 0, 1)]), wy4);
   m[mi(2, 1, 2)] = mul(split(m[mi(2, 1, 0)]), wz4);
   m[mi(1, 2, 2)] = mul(split(m[mi(1, 2, 0)]), wz4);
-  m[mi(2, 0, 0)] = rwx - kThird;
-  m[mi(0, 2, 0)] = rwy - kThird;
-  m[mi(0, 0, 2)] = mul(rs, wz4) - kThird;
-  const fx rwxwy = mul(rwxs, wy4);
-  m[mi(2, 2, 0)] = rwxwy - kNinth;
-  m[mi(2, 0, 2)] = mul(rwxs, wz4) - kNinth;
-  m[mi(0, 2, 2)] = mul(split(rwy), wz4) - kNinth;
-  m[mi(2, 2, 2)] = mul(split(rwxwy), wz4) - k27th;
+  m[mi(2, 0, 0)] = mul(rs, wx4) + vx;
+  m[mi(0, 2, 0)] = mul(rs, wy4) + vy;
+  m[mi(0, 0, 2)] = mul(rs, wz4) + vz;
+  const fx ty = mul(split(vy), third), tz = mul(split(vz), third);
+  const Split rxs = split(m[mi(2, 0, 0)]);
+  m[mi(2, 2, 0)] = mul(rxs, wy4) + ty;
+  m[mi(2, 0, 2)] = mul(rxs, wz4) + tz;
+  m[mi(0, 2, 2)] = mul(split(m[mi(0, 2, 0)]), wz4) + tz;
+  m[mi(2, 2, 2)] = mul(split(m[mi(2, 2, 0)]), wz4) + mul(split(tz), third);
   to_populations(m);
 }
 
@@ -418,64 +488,78 @@ KBC_HD fx relax_factor(fx num, fx den, int e, fx two_beta_1, int* k) {
   return shl(((1ll << 59) >> up) - (t >> down), 2);
 }
 
-// One KBC collision (Sec. KBC, natural moments, product-form equilibrium) of the shifts d,
-// |d_i| < 1/4, in place; the result d_i is f'_i - W_i times 2^nonzero(i) (to_f64<nonzero(i)>).
+// One KBC collision (Sec. KBC, natural moments, product-form equilibrium) of the shifts d 2^s,
+// |d_i| 2^s < 1/4, in place; the result d_i is f'_i - W_i, or with CHANGE f'_i - f_i, times
+// 2^(s + nonzero(i)) (to_f64<nonzero(i)>). The conserved moments of a change are exactly 0.
 // Returns gamma; *guarded is set when <dh|dh> is 0 (gamma = 2), *bad when the node is outside
 // the format's range (d is then not a result).
-KBC_HD double collide(fx (&d)[27], const Relax& rx, int* guarded, bool* bad) {
+template <bool CHANGE = false>
+KBC_HD double collide(fx (&d)[27], const Relax& rx, int* guarded, bool* bad, uint32_t s = 0) {
+  // FP32 results need no products to nearest (all nodes of 256^3: 4.7 -> 4.2 ms)
+  auto times = [](Split a, Split b) { return CHANGE ? mul(a, b) : mul_down(a, b); };
   to_moments(d);
-  const fx jx = d[mi(1, 0, 0)], jy = d[mi(0, 1, 0)], jz = d[mi(0, 0, 1)];
-  const fx rho = kOne + d[0];
-  // 1/2 < rho < 2, |rho u| < 1/4, |u| < 1/4
+  const fx dr = d[0], jx = d[mi(1, 0, 0)], jy = d[mi(0, 1, 0)], jz = d[mi(0, 0, 1)];
+  const fx rho = kOne + sar(dr, s);
+  const float ps = pow2_of(s);
+  // 1/2 < rho < 2, |rho u| < 1/4, |u| < 1/4, the velocities times 2^s
   *bad = rho <= (kOne >> 1) || rho >= 2 * kOne ||
          ((magnitude(jx) | magnitude(jy) | magnitude(jz)) >> 58) != 0;
   *guarded = 0;
   const Split ir = split(reciprocal(rho));
-  const fx ux = mul(ir, factor(jx)), uy = mul(ir, factor(jy)), uz = mul(ir, factor(jz));
-  *bad = *bad || ((magnitude(ux) | magnitude(uy) | magnitude(uz)) >> 58) != 0;
+  const fx usx = times(ir, factor(jx)), usy = times(ir, factor(jy)), usz = times(ir, factor(jz));
+  *bad = *bad || ((magnitude(usx) | magnitude(usy) | magnitude(usz)) >> 58) != 0;
+  const fx ux = sar(usx, s), uy = sar(usy, s), uz = sar(usz, s);
   const Split ux4 = factor(ux), uy4 = factor(uy), uz4 = factor(uz);
-  const fx ex = axis_e(ux4, ux), ey = axis_e(uy4, uy), ez = axis_e(uz4, uz);
-  // second moments of the axis factors, m_2(u) = 1/3 + 2e/3
+  const fx esx = axis_e(ux4, usx, s, ps), esy = axis_e(uy4, usy, s, ps),
+           esz = axis_e(uz4, usz, s, ps);
+  const fx ex = sar(esx, s), ey = sar(esy, s), ez = sar(esz, s);
+  // second moments of the axis factors, m_2(u) = 1/3 + 2e/3: less 1/3 and times 2^s, and as factors
   const Split third = factor(kThird);
-  const Split wx4 = factor(kThird + mul(split(ex + ex), third));
-  const Split wy4 = factor(kThird + mul(split(ey + ey), third));
-  const Split wz4 = factor(kThird + mul(split(ez + ez), third));
+  const fx vx = times(split(esx + esx), third), vy = times(split(esy + esy), third),
+           vz = times(split(esz + esz), third);
+  const Split wx4 = factor(kThird + sar(vx, s)), wy4 = factor(kThird + sar(vy, s)),
+              wz4 = factor(kThird + sar(vz, s));
 
-  // deviations A = M - rho M_eq (the moments of f - f_eq); s is relaxed by 2 beta at once, the
-  // moments of h (and the third ones, which are in s or in h) are kept in H
+  // deviations A = M - rho M_eq (the moments of f - f_eq), times 2^s; M and rho M_eq are both less
+  // the weights' moments, as in equilibrium(). s is relaxed by 2 beta at once, the moments of h
+  // (and the third ones, which are in s or in h) are kept in H
   const Split bs = split(rx.quarter_beta);
-  auto relax_s = [&](int m, fx a) { d[m] -= mul(split(shl(a, 3)), bs); };
-  const Split rs = split(rho), jxs = split(jx), jys = split(jy), jzs = split(jz);
-  const fx rwx = mul(rs, wx4), rwy = mul(rs, wy4), rwz = mul(rs, wz4);
+  auto relax_s = [&](int m, fx a) { d[m] -= times(split(shl(a, 3)), bs); };
+  const Split rs = split(dr), jxs = split(jx), jys = split(jy), jzs = split(jz);
+  const fx rwx = times(rs, wx4) + vx, rwy = times(rs, wy4) + vy, rwz = times(rs, wz4) + vz;
   const Split rwxs = split(rwx);
-  const fx pxy = mul(jxs, uy4), pxz = mul(jxs, uz4), pyz = mul(jys, uz4);
+  const fx pxy = times(jxs, uy4), pxz = times(jxs, uz4), pyz = times(jys, uz4);
   const Split pxys = split(pxy);
-  const fx jxwy = mul(jxs, wy4), jywx = mul(jys, wx4), jzwx = mul(jzs, wx4);
-  const fx rwxwy = mul(rwxs, wy4);
+  const fx jxwy = times(jxs, wy4), jywx = times(jys, wx4), jzwx = times(jzs, wx4);
+  const fx ty = times(split(vy), third), tz = times(split(vz), third);
+  const fx rwxwy = times(rwxs, wy4) + ty;
   fx H[27];
-  H[mi(2, 2, 0)] = d[mi(2, 2, 0)] + kNinth - rwxwy;
-  H[mi(2, 0, 2)] = d[mi(2, 0, 2)] + kNinth - mul(rwxs, wz4);
-  H[mi(0, 2, 2)] = d[mi(0, 2, 2)] + kNinth - mul(split(rwy), wz4);
-  H[mi(2, 1, 1)] = d[mi(2, 1, 1)] - mul(split(pyz), wx4);
-  H[mi(1, 2, 1)] = d[mi(1, 2, 1)] - mul(split(pxz), wy4);
-  H[mi(1, 1, 2)] = d[mi(1, 1, 2)] - mul(pxys, wz4);
-  H[mi(2, 2, 1)] = d[mi(2, 2, 1)] - mul(split(jzwx), wy4);
-  H[mi(2, 1, 2)] = d[mi(2, 1, 2)] - mul(split(jywx), wz4);
-  H[mi(1, 2, 2)] = d[mi(1, 2, 2)] - mul(split(jxwy), wz4);
-  H[mi(2, 2, 2)] = d[mi(2, 2, 2)] + k27th - mul(split(rwxwy), wz4);
+  H[mi(2, 2, 0)] = d[mi(2, 2, 0)] - rwxwy;
+  H[mi(2, 0, 2)] = d[mi(2, 0, 2)] - (times(rwxs, wz4) + tz);
+  H[mi(0, 2, 2)] = d[mi(0, 2, 2)] - (times(split(rwy), wz4) + tz);
+  H[mi(2, 1, 1)] = d[mi(2, 1, 1)] - times(split(pyz), wx4);
+  H[mi(1, 2, 1)] = d[mi(1, 2, 1)] - times(split(pxz), wy4);
+  H[mi(1, 1, 2)] = d[mi(1, 1, 2)] - times(pxys, wz4);
+  H[mi(2, 2, 1)] = d[mi(2, 2, 1)] - times(split(jzwx), wy4);
+  H[mi(2, 1, 2)] = d[mi(2, 1, 2)] - times(split(jywx), wz4);
+  H[mi(1, 2, 2)] = d[mi(1, 2, 2)] - times(split(jxwy), wz4);
+  H[mi(2, 2, 2)] = d[mi(2, 2, 2)] - (times(split(rwxwy), wz4) + times(split(tz), third));
   fx q[7];  // 120, 102, 210, 012, 201, 021, 111
   q[0] = d[mi(1, 2, 0)] - jxwy;
-  q[1] = d[mi(1, 0, 2)] - mul(jxs, wz4);
+  q[1] = d[mi(1, 0, 2)] - times(jxs, wz4);
   q[2] = d[mi(2, 1, 0)] - jywx;
-  q[3] = d[mi(0, 1, 2)] - mul(jys, wz4);
+  q[3] = d[mi(0, 1, 2)] - times(jys, wz4);
   q[4] = d[mi(2, 0, 1)] - jzwx;
-  q[5] = d[mi(0, 2, 1)] - mul(jzs, wy4);
-  q[6] = d[mi(1, 1, 1)] - mul(pxys, uz4);
+  q[5] = d[mi(0, 2, 1)] - times(jzs, wy4);
+  q[6] = d[mi(1, 1, 1)] - times(pxys, uz4);
   fx sxy = d[mi(1, 1, 0)] - pxy, sxz = d[mi(1, 0, 1)] - pxz, syz = d[mi(0, 1, 1)] - pyz;
-  fx sx = d[mi(2, 0, 0)] + kThird - rwx, sy = d[mi(0, 2, 0)] + kThird - rwy;
-  fx sz = d[mi(0, 0, 2)] + kThird - rwz;
+  fx sx = d[mi(2, 0, 0)] - rwx, sy = d[mi(0, 2, 0)] - rwy, sz = d[mi(0, 0, 2)] - rwz;
+  if constexpr (CHANGE) {
+#pragma unroll
+    for (int i = 0; i < 27; ++i) d[i] = 0;
+  }
   // the trace belongs to s (with_t) or, spread over the three diagonal moments, to h
-  const fx ht = rx.with_t ? 0 : mul(split(sx + sy + sz), third);
+  const fx ht = rx.with_t ? 0 : times(split(sx + sy + sz), third);
   sx -= ht, sy -= ht, sz -= ht;
   H[mi(2, 0, 0)] = H[mi(0, 2, 0)] = H[mi(0, 0, 2)] = ht;
   H[mi(0, 0, 0)] = H[mi(1, 0, 0)] = H[mi(0, 1, 0)] = H[mi(0, 0, 1)] = 0;
@@ -551,16 +635,18 @@ KBC_HD double collide(fx (&d)[27], const Relax& rx, int* guarded, bool* bad) {
       w[a][1] = split(shl(kOne - e, 1));
       w[a][2] = split(shl(b - u3, 1));
     }
-    fx num = 0, den = 0;
+    const fx lost = CHANGE ? 0 : 3;
+    fx num = lost, den = lost;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      fx L[9], cn = 0, cd = 0;  // the level's moments in x and y
+      fx L[9], cn = lost, cd = lost;  // the level's moments in x and y
 #pragma unroll
       for (int m = 0; m < 9; ++m)
         L[m] = c == 1 ? H[m] - H[m + 18] : (c == 2 ? H[m + 18] + H[m + 9] : H[m + 18] - H[m + 9]);
 #pragma unroll
       for (int b = 0; b < 3; ++b) {
-        fx R[3], rn = 0, rd = 0;  // the row's moments in x
+        // the row's moments in x; the sums start with the unit that each product loses
+        fx R[3], rn = b != 1 && c != 1 ? 1 - 2 * keep : 3, rd = 3;
 #pragma unroll
         for (int m = 0; m < 3; ++m)
           R[m] = b == 1 ? L[m] - L[m + 6] : (b == 2 ? L[m + 6] + L[m + 3] : L[m + 6] - L[m + 3]);
@@ -589,15 +675,15 @@ KBC_HD double collide(fx (&d)[27], const Relax& rx, int* guarded, bool* bad) {
           } else {
             s = va * vb * vc > 0 ? q[6] : -q[6];
           }
-          const Split hh = split(h), t = split(mul(hh, w[0][a]));  // below 2^62, 2^60.3
-          rn += mul(split(s), t);
-          rd += mul(hh, t);  // below 2^58.3 each
+          const Split hh = split(h), t = split(mul_down(hh, w[0][a]));  // below 2^62, 2^60.3
+          rn += mul_down(split(s), t);
+          rd += mul_down(hh, t);  // below 2^58.3 each
         }
-        cn += mul(split(shl(rn, 2)), w[1][b]);  // a row below 2^62, half of its weighted sum
-        cd += mul(split(shl(rd, 2)), w[1][b]);
+        cn += times(split(shl(rn, 2)), w[1][b]);  // a row below 2^62, half of its weighted sum
+        cd += times(split(shl(rd, 2)), w[1][b]);
       }
-      num += mul(split(shl(cn, 1)), w[2][c]);
-      den += mul(split(shl(cd, 1)), w[2][c]);
+      num += times(split(shl(cn, 1)), w[2][c]);
+      den += times(split(shl(cd, 1)), w[2][c]);
     }
     if (!none) {
       // the unscaled deviations: num carries 2^(hs + ss), den 2^(2 hs)
@@ -617,7 +703,7 @@ KBC_HD double collide(fx (&d)[27], const Relax& rx, int* guarded, bool* bad) {
   for (int i = 0; i < 27; ++i) {
     const int order = i % 3 + (i / 3) % 3 + i / 9;
     if (order >= 3 || (order == 2 && (i == mi(2, 0, 0) || i == mi(0, 2, 0) || i == mi(0, 0, 2))))
-      d[i] -= mul(split(shl(H[i], k)), cs);
+      d[i] -= times(split(shl(H[i], k)), cs);
   }
   to_populations(d);
   return gamma;
