@@ -678,25 +678,7 @@ static __global__ void gap_final_kernel(const double* partials, int nblocks, dou
 }
 
 // ------------------------------------------------------------------ density pre-solve
-// rho - 1 of 27 stored shifts, for the density change of the pre-solve: both its kernels take it
-// from here, so that a fixed point gives exactly 0. FP64: summed in fixed point (v receives the
-// shifts; *in_range says that they and the sum fit), FP64 sums otherwise.
-__device__ __forceinline__ double presolve_drho(const double (&d)[27], fix::fx (&v)[27],
-                                                fix::fx* sum, bool* in_range) {
-  uint32_t top = 0;
-#pragma unroll
-  for (int i = 0; i < 27; ++i) v[i] = fix::from_f64(d[i], &top);
-  fix::fx s = 0;
-#pragma unroll
-  for (int i = 0; i < 27; ++i) s += v[i];
-  *sum = s;
-  *in_range = top < fix::kTopF64 && s > -(fix::kOne >> 2) && s < (fix::kOne >> 2);
-  if (*in_range) return fix::to_f64<0>(s);
-  double t = 0.0;
-#pragma unroll
-  for (int i = 0; i < 27; ++i) t += d[i];
-  return t;
-}
+// rho - 1 of 27 stored shifts, for the density change of the pre-solve
 __device__ __forceinline__ float presolve_drho(const float (&d)[27]) {
   float s = 0.0f;
 #pragma unroll
@@ -704,9 +686,10 @@ __device__ __forceinline__ float presolve_drho(const float (&d)[27]) {
   return s;
 }
 __device__ __forceinline__ double presolve_drho(const double (&d)[27]) {
-  fix::fx v[27], s;
+  fix::fx v[27], sum;
+  uint32_t s, top;
   bool in_range;
-  return presolve_drho(d, v, &s, &in_range);
+  return fix::presolve_density(d, v, &sum, &s, &top, &in_range);
 }
 
 // One iteration of the consistent-initialisation loop (Sec. "Numerical Simulations", after
@@ -774,8 +757,8 @@ __device__ __noinline__ void presolve_node_fp64(const double* src, double* dst, 
 
 // The FP64 pre-solve step in fixed point (kbc_fix.cuh), one node per thread over the node order;
 // nodes outside the format's range are stepped in FP64. FULL: beta2 = 1, the default relaxation,
-// sets f to f_eq, so that the populations are only summed. 100^3 AA: 564 -> 114 us an iteration
-// (456 B a node: 68 us), 120 for a general beta2; bound by the integer pipe (FP64: by the FP64
+// sets f to f_eq, so that the populations are only summed. 100^3 AA: 564 -> 117 us an iteration
+// (456 B a node: 68 us), 141 for a general beta2; bound by the integer pipe (FP64: by the FP64
 // pipe, ~190 operations a node).
 template <int MODE, bool FULL>
 __global__ void __maxnreg__(128) presolve_fix_kernel(const double* src, double* dst, Geo g,
@@ -797,30 +780,11 @@ __global__ void __maxnreg__(128) presolve_fix_kernel(const double* src, double* 
     d[I] = src[(uint64_t)Pat::load_plane(I) * g.P + nb.template at<I, Pat::load_shift>()];
   });
   const double ux = u0[n], uy = u0[g.P + n], uz = u0[2 * g.P + n];
-  fix::fx v[27], p[27], sum;
-  bool ok;
-  const double drho = presolve_drho(d, v, &sum, &ok);
+  fix::fx p[27];
+  uint32_t sc;
+  double drho;
+  const bool ok = fix::presolve<FULL>(d, ux, uy, uz, beta2, p, &sc, &drho);
   if (store) rho_prev[n] = (float)drho;
-  uint32_t top = 0;
-  const fix::fx u[3] = {fix::from_f64(ux, &top), fix::from_f64(uy, &top), fix::from_f64(uz, &top)};
-  ok = ok && top < fix::kTopF64;
-  if (ok) {
-    fix::equilibrium(sum, u[0], u[1], u[2], p);
-    if constexpr (!FULL) {
-      // f - beta2 (f - f_eq), populations times 2^N: beta2 / 8 < 1/4 as a factor of 2^64
-      const fix::Split b = fix::split((fix::fx)(beta2 * 2305843009213693952.0));
-      uint32_t far = 0;
-      Unroll<0, 27>::run([&](auto ic) {
-        constexpr int I = decltype(ic)::value;
-        v[I] = fix::shl(v[I], fix::nonzero(I));
-        p[I] = v[I] - p[I];
-        far |= fix::high(p[I]);
-      });
-      ok = (far >> 27) == 0;  // |f - f_eq| 2^N < 1/2
-#pragma unroll
-      for (int i = 0; i < 27; ++i) p[i] = v[i] - fix::mul(fix::split(fix::shl(p[i], 3)), b);
-    }
-  }
   if (!ok) {
     presolve_node_fp64<MODE>(src, dst, g, beta2, ux, uy, uz, x, y, z);
     return;
@@ -828,7 +792,7 @@ __global__ void __maxnreg__(128) presolve_fix_kernel(const double* src, double* 
   Unroll<0, 27>::run([&](auto ic) {
     constexpr int I = decltype(ic)::value;
     dst[(uint64_t)Pat::store_plane(I) * g.P + nb.template at<I, Pat::store_shift>()] =
-        fix::to_f64<fix::nonzero(I)>(p[I]);
+        fix::to_f64<fix::nonzero(I)>(p[I], sc);
   });
 }
 

@@ -709,5 +709,87 @@ KBC_HD double collide(fx (&d)[27], const Relax& rx, int* guarded, bool* bad, uin
   return gamma;
 }
 
+// ------------------------------------------------------------------ density pre-solve
+// rho - 1 of the shifts d, for the pre-solve and the measure of its change, which both take it from
+// here. In fixed point: v receives the shifts (times 2^s), *sum their sum, *in_range says that they
+// fit (the sum below 1/4, which that of a density shift is: 27/8 of the largest); FP64 sums otherwise.
+KBC_HD double presolve_density(const double (&d)[27], fx (&v)[27], fx* sum, uint32_t* s,
+                               uint32_t* top, bool* in_range) {
+  *top = 0;
+#pragma unroll
+  for (int i = 0; i < 27; ++i) *top = top_of(d[i]) > *top ? top_of(d[i]) : *top;
+  *in_range = scale_to<double, 4>(*top, s) && *top < kTopF64;
+#pragma unroll
+  for (int i = 0; i < 27; ++i) v[i] = scaled(d[i], *s);
+  fx a = 0;
+#pragma unroll
+  for (int i = 0; i < 27; ++i) a += v[i];
+  *sum = a;
+  *in_range = *in_range && a > -(kOne >> 2) && a < (kOne >> 2);
+  if (*in_range) return to_f64<0>(a, *s);
+  double t = 0.0;
+#pragma unroll
+  for (int i = 0; i < 27; ++i) t += d[i];
+  return t;
+}
+
+// One node of the pre-solve: p = f - beta2 (f - f_eq(rho(f), u)), times 2^(s + nonzero(i)); FULL:
+// beta2 = 1, so that p is f_eq. What is stored is what the next iteration reads: the populations
+// are rounded to units of the grid that it reads the shifts in, or to 53 bits of their class's
+// largest and of the one at rest, so that the conversion to FP64 is exact, and the one at rest takes
+// what that leaves of the density: the sum of what is read is the density again, to the bit. Otherwise the residues of the
+// roundings, the same in every iteration of a settled node, add up in the density. *drho receives
+// rho - 1 of d. False: not in the range.
+template <bool FULL>
+KBC_HD bool presolve(const double (&d)[27], double ux, double uy, double uz, double beta2,
+                     fx (&p)[27], uint32_t* s, double* drho) {
+  fx v[27], dr;
+  uint32_t top, sd;
+  bool ok;
+  *drho = presolve_density(d, v, &dr, &sd, &top, &ok);
+  // the velocity's scale, if smaller: |u| 2^s < 1/4
+  const uint32_t tx = top_of(ux), ty = top_of(uy), tz = top_of(uz);
+  uint32_t tu = tx > ty ? tx : ty, su;
+  tu = tz > tu ? tz : tu;
+  scale_to<double, 2>(tu, &su);
+  *s = top == 0 || (su < sd && tu != 0) ? su : sd;
+  ok = ok && tu < kTopF64 && *s <= kMaxScale;
+  if (!ok) return false;
+  const uint32_t less = sd > *s ? sd - *s : 0;
+  dr = sar(dr, less);
+  equilibrium(dr, scaled(ux, *s), scaled(uy, *s), scaled(uz, *s), p, *s);
+  if constexpr (!FULL) {
+    // f - beta2 (f - f_eq): beta2 / 8 < 1/4 as a factor of 2^64
+    const Split b = split((fx)(beta2 * 2305843009213693952.0));
+    uint32_t far = 0;
+#pragma unroll
+    for (int i = 0; i < 27; ++i) {
+      v[i] = shl(sar(v[i], less), nonzero(i));
+      p[i] = v[i] - p[i];
+      far |= high(p[i]);
+    }
+    ok = (far >> 27) == 0;  // |f - f_eq| 2^N < 1/2
+#pragma unroll
+    for (int i = 0; i < 27; ++i) p[i] = v[i] - mul(split(shl(p[i], 3)), b);
+  }
+  uint32_t most[4] = {0, 0, 0, 0};
+#pragma unroll
+  for (int i = 0; i < 27; ++i) most[nonzero(i)] |= high(p[i]);
+#pragma unroll
+  for (int i = 0; i < 27; ++i) {
+    const int N = nonzero(i);
+    if (N == 0) continue;
+    // bits above 53
+    const int rest = 11 - clz32(most[0]), own = 11 - clz32(most[N]) - N;
+    const int over = own > rest ? own : rest;
+    const uint32_t n = N + (over > 0 ? over : 0);
+    const fx q = sar(p[i] + (fx)(1ull << (n - 1)), n);  // to nearest
+    dr -= shl(q, n - N);
+    p[i] = shl(q, n);
+  }
+  p[13] = dr;
+  return ok;
+}
+
 }  // namespace fix
 }  // namespace kbc

@@ -1,5 +1,5 @@
-"""The fixed-point collision (csrc/kbc_fix.cuh), compiled for the host, at every
-amplitude of the flow: relative to the node's shifts it must be no less exact than the same in
+"""The fixed-point collision and pre-solve (csrc/kbc_fix.cuh), compiled for the host, at every
+amplitude of the flow: relative to the node's shifts they must be no less exact than the same in
 FP64 instructions, and over many steps mass and momentum must drift no more."""
 import ctypes
 import os
@@ -71,6 +71,29 @@ extern "C" void collide32(int n, const float* f, double* o, int* flags, double b
     flags[k] = (bad ? 2 : 0) | gd;
     for (int i = 0; i < 27; ++i) o[k * 27 + i] = value(v[i], i, s);
   }
+}
+// `iters` pre-solve iterations of each node by itself (a uniform flow); rho - 1 of the states
+// before the last and after it
+extern "C" int presolve(int n, int iters, double* d, const double* u, double* before,
+                        double* after, double beta2) {
+  int bad = 0;
+  for (int k = 0; k < n; ++k) {
+    double(&f)[27] = *(double(*)[27])(d + 27 * k);
+    for (int t = 0; t < iters; ++t) {
+      fix::fx p[27];
+      uint32_t s;
+      const double* w = u + 3 * k;
+      const bool ok = beta2 == 1.0 ? fix::presolve<true>(f, w[0], w[1], w[2], beta2, p, &s, before + k)
+                                   : fix::presolve<false>(f, w[0], w[1], w[2], beta2, p, &s, before + k);
+      if (!ok) { ++bad; break; }
+      for (int i = 0; i < 27; ++i) f[i] = value(p[i], i, s);
+    }
+    fix::fx v[27], sum;
+    uint32_t s, top;
+    bool in;
+    after[k] = fix::presolve_density(f, v, &sum, &s, &top, &in);
+  }
+  return bad;
 }
 '''
 
@@ -252,3 +275,40 @@ def test_edges_of_the_scale(lib):
     assert fl.tolist() == [1, 2, 0, 0, 0] and not o[0].any()
     ref, _ = reference(f[2:], beta, 1, 1, 0, LD)
     assert np.abs((o[2:] - ref) / size).max() <= 2 * 27 * 2.0 ** -54
+
+
+@pytest.mark.parametrize("amp", [0.03, 1e-2, 1e-4, 1e-6, 1e-8, 1e-12])
+@pytest.mark.parametrize("beta2", [1.0, 2 / 1.6, 2 / 1.12, 0.4])
+def test_presolve_of_uniform_flow_settles(lib, amp, beta2):
+    """The measured change of the density is exactly 0, and the density stays where it was."""
+    rng = np.random.default_rng(6)
+    n = 40
+    u = np.concatenate([np.array([[3.0, -2.0, 1.0]]), rng.uniform(-3, 3, (n - 1, 3))]) * amp
+    u[5:10, 1] = 0
+    u = np.ascontiguousarray(u)
+    drho = np.where(np.arange(n) % 2, amp * rng.uniform(-1, 1, n), 0).astype(LD)
+    d = equilibrium(drho, u.T.astype(LD), LD).astype(np.float64)
+    before, after = np.empty(n), np.empty(n)
+    start = d.copy()
+    bad = lib.presolve(n, 200, ptr(d), ptr(u), ptr(before), ptr(after), ctypes.c_double(beta2))
+    assert bad == 0
+    assert np.array_equal(before, after)
+    size = np.abs(start).max(1)
+    assert (np.abs((d - start).astype(LD).sum(1)) / size).max() <= 27 * 2.0 ** -53
+    assert (np.abs(d - start).max(1) / size).max() <= 27 * 2.0 ** -53
+
+
+@pytest.mark.parametrize("amp", [0.1, 1e-2, 1e-4, 1e-8])
+def test_presolve_error_is_that_of_fp64(lib, amp):
+    """One iteration at the default relaxation: f_eq as exact as in FP64 instructions."""
+    rng = np.random.default_rng(7)
+    n = 2000
+    u = np.ascontiguousarray(amp * rng.uniform(-1, 1, (n, 3)))
+    d = equilibrium((amp / 4 * rng.uniform(-1, 1, n)).astype(LD), u.T.astype(LD), LD)
+    d = d.astype(np.float64)
+    ref = equilibrium(d.astype(LD).sum(1), u.T.astype(LD), LD)
+    f64 = equilibrium(d.sum(1), u.T, np.float64)
+    before, after = np.empty(n), np.empty(n)
+    size = np.abs(d).max(1, keepdims=True).astype(LD)
+    assert lib.presolve(n, 1, ptr(d), ptr(u), ptr(before), ptr(after), ctypes.c_double(1.0)) == 0
+    assert rms((d - ref) / size) <= rms((f64 - ref) / size)
