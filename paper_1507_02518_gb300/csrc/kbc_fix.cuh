@@ -265,15 +265,16 @@ template <int N> KBC_HD float to_f32(fx v) {
   const uint32_t r = t == 0 ? 0 : b + ((uint32_t)(32 - kFrac - N - lz) << 23);
   return f32_of(r | ((uint32_t)((uint64_t)v >> 32) & 0x80000000u));
 }
-// The same towards zero with the last bit set (0 stays 0), for a further rounding to a shorter
-// type, which then rounds v (a tie of it away from zero) as long as it has at most 22 bits of v
-// from 2^16 units, 2^-44, on. |v| < 2^63. FP16 initialisation of 256^3: 1.08 -> 0.79 ms.
+// The same rounded to odd: towards zero, with the last bit set where that is not exact, for a
+// further rounding to a shorter type, which then rounds v itself, ties to even, as long as it has at
+// most 22 bits of v from 2^16 units, 2^-44, on. |v| < 2^63. FP16 initialisation of 256^3: 1.08 ->
+// 0.87 ms.
 template <int N> KBC_HD float to_f32_odd(fx v) {
-  const int32_t hi = (int32_t)((uint64_t)v >> 32);
-  const float f = add_rz<20 + N>((float)(hi >> 8),
-                                 mulf(window<16>(v, ((uint32_t)v & 0xffffu) != 0),
-                                      1.0f / (float)(1ull << (44 + N))));
-  return f32_of(bits_of(f) | (v != 0 ? 1u : 0u));
+  const float a = (float)((int32_t)((uint64_t)v >> 32) >> 8);
+  const float b = mulf(window<16>(v, ((uint32_t)v & 0xffffu) != 0), 1.0f / (float)(1ull << (44 + N)));
+  const float f = add_rz<20 + N>(a, b);
+  const float part = add_rn<20 + N>(-a, f);  // exact: what f holds of b
+  return f32_of(bits_of(f) | (part != b ? 1u : 0u));
 }
 
 // ------------------------------------------------------------------ products
