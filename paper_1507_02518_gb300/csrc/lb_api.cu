@@ -1599,19 +1599,18 @@ lb_status lb_batch_diagnostics(lb_batch* b, lb_diag* out) {
     const uint64_t room = b->views[0]->stage_nodes * 27 / kbc::kDiagSums;
     std::vector<double> sums;
     for (int k0 = 0; k0 < b->nbox;) {
-      const int n = (int)std::min<uint64_t>((uint64_t)(b->nbox - k0), room);
+      int n = (int)std::min<uint64_t>((uint64_t)(b->nbox - k0), room);
       double* dev = b->views[0]->staging;
+      lb_status stop = LB_OK;  // a box that refuses ends the call, after the boxes before it
       for (int k = 0; k < n; ++k) {
-        lb_ctx* v = b->views[k0 + k];
-        lb_status s = enqueue_diag(v, dev + (size_t)k * kbc::kDiagSums);
-        if (s != LB_OK) {
-          b->err = "box " + std::to_string(k0 + k) + ": " + v->err;
-          return s;
-        }
+        stop = enqueue_diag(b->views[k0 + k], dev + (size_t)k * kbc::kDiagSums);
+        if (stop != LB_OK) n = k;
       }
       sums.resize((size_t)n * kbc::kDiagSums);
-      cudaError_t e = cudaMemcpyAsync(sums.data(), dev, sums.size() * sizeof(double),
-                                      cudaMemcpyDeviceToHost, b->stream);
+      cudaError_t e = cudaSuccess;
+      if (n > 0)
+        e = cudaMemcpyAsync(sums.data(), dev, sums.size() * sizeof(double),
+                            cudaMemcpyDeviceToHost, b->stream);
       if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
       if (e != cudaSuccess)
         return bfail(b, LB_ERR_CUDA, std::string("diagnostics: ") + cudaGetErrorString(e));
@@ -1623,6 +1622,10 @@ lb_status lb_batch_diagnostics(lb_batch* b, lb_diag* out) {
         if (s != LB_OK && s != LB_ERR_NONFINITE) return s;
       }
       k0 += n;
+      if (stop != LB_OK) {
+        b->err = "box " + std::to_string(k0) + ": " + b->views[k0]->err;
+        return stop;
+      }
     }
     return worst;
   });
