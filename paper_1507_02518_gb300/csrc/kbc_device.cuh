@@ -1376,6 +1376,18 @@ template <> struct Pattern<MODE_AA_ODD> {
   __host__ __device__ static constexpr int store_plane(int i) { return i; }
 };
 
+// Where plane `plane` holds what node n loads from it, for every n that is not at an edge of the box in
+// x or y (x shifts left out): a node of the box for every n of the box.
+template <int MODE> __host__ __device__ inline uint64_t ahead_node(const Geo& g, uint32_t plane,
+                                                                   uint64_t n) {
+  if (MODE == MODE_AA_EVEN) return n;
+  // the plane's own velocity: a pull step loads plane i at -v_i, an odd AA step plane 26 - i there
+  const int y = (int)(plane / 3 % 3) - 1, z = (int)(plane / 9) - 1;
+  const int64_t o = y * (int64_t)g.nx + z * (int64_t)g.nxy;
+  const int64_t m = (int64_t)n + (MODE == MODE_PULL ? -o : o);
+  return (uint64_t)(m < 0 ? m + (int64_t)g.P : (m >= (int64_t)g.P ? m - (int64_t)g.P : m));
+}
+
 // One node loaded, collided in FP64 instructions (collide<double>, with the oracle's guard) and
 // stored, where the step's pattern keeps its inputs and outputs: the form for nodes that the
 // fixed-point collision does not take. The inputs are still there (pull: src, which a step does

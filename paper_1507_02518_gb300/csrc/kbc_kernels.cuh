@@ -104,31 +104,34 @@ __device__ __forceinline__ void advance_node(uint32_t& x, uint32_t& y, uint32_t&
 }
 
 // Brings into L2 what the blocks one wave ahead will load (kWave blocks are resident on the
-// chip: 3 on each of 152 SMs): the warp's share of the 27 planes of the tile that starts kWave
-// blocks after node n, a 128-byte line per lane. With 12 warps per SM the loads' latency is what
-// the step waits for. us a step without -> with: adjacent pairs FP16 256^3 AA 411 -> 378, pull 383
-// -> 367, 200^3 AA 229 -> 193, FP32 AA 256^3 551 -> 534, 200^3 (node order) 321 -> 264; pairs
-// (n, n + 32) FP32 201^3 AA 321 -> 293, pull 292 -> 287, FP16 269 -> 241, 243 -> 218, central moments
-// FP32 192^3 pull 268 -> 257. The adjacent-pair FP32 pull step, at the DRAM rate already, lost
-// (537 -> 560) and does without. (200 or 912 blocks ahead: FP16 AA 391, 390. Loading the next tile
-// into registers instead takes 238 of them, 8 warps per SM: 438.)
+// chip: 3 on each of 152 SMs): of each of the 27 planes the warp's share of the tile that starts
+// kWave blocks after node n, moved by the plane's velocity as the step's loads are (ahead_node()), a
+// 128-byte line per lane. With 12 warps per SM the loads' latency is what the step waits for. us a
+// step without -> with: adjacent pairs FP16 256^3 AA 422 -> 387, pull 413 -> 384, FP32 AA 256^3 550 ->
+// 540, 768^3 14722 -> 14336, 1536 x 768 x 192 7361 -> 7134; pairs (n, n + 32) FP32 201^3 AA 325 -> 304,
+// pull 293 -> 289, central moments FP32 pull 192^3 271 -> 260, 384^3 2130 -> 2030. (Lines of the same
+// node in every plane, without the move, are read after their use where a plane of the box is larger
+// than a wave's nodes: 1536 x 768 x 192 FP32 AA 8146.) The adjacent-pair FP32 pull step, at the DRAM
+// rate already, lost (256^3 537 -> 555) and does without. (200 or 912 blocks ahead: FP16 AA 391, 390
+// where 456 took 378. Loading the next tile into registers instead takes 238 of them, 8 warps per SM:
+// 438.)
 constexpr uint32_t kWave = 456;
-template <typename S>
+template <typename S, int MODE>
 __device__ __forceinline__ void prefetch_ahead(const S* src, const Geo& g, uint64_t n) {
   const uint32_t lane = threadIdx.x & 31;
   n += (uint64_t)kWave * 2 * blockDim.x + 2 * (threadIdx.x & ~31u);
   if (lane < 27 && n < g.P) {
+    n = ahead_node<MODE>(g, lane, n);
     const S* p = src + (uint64_t)lane * g.P + n;
     asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
     // FP32: the second half of the warp's 64 nodes
     if (sizeof(S) == 4 && n + 32 < g.P) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + 32));
   }
 }
-// where it is worth its instructions: populations larger than L2 (129 MB), of up to 40 GB (FP32 AA
-// without -> with: 640^3 9420 -> 9261 us, 704^3 (38 GB) 11977 -> 11841, 768^3 (49 GB) 14666 -> 15012)
-template <typename S> __host__ __device__ inline bool beyond_l2(const Geo& g) {
-  const uint64_t bytes = 27 * g.P * sizeof(S);
-  return bytes > (129ull << 20) && bytes <= 40000000000ull;
+// where it is worth its instructions: a step's populations (pull: both buffers) larger than L2
+// (129 MB); FP16 pull 112^3 41.5 -> 38.4 us, 128^3 54.4 -> 50.8
+template <typename S, int MODE> __host__ __device__ inline bool beyond_l2(const Geo& g) {
+  return 27 * g.P * sizeof(S) * (MODE == MODE_PULL ? 2 : 1) > (129ull << 20);
 }
 
 // Two nodes per thread with packed FP32x2 arithmetic: a block of up to 128 threads covers
@@ -142,7 +145,7 @@ __global__ void __launch_bounds__(128, 3) pair_step_kernel(const S* src, S* dst,
   const uint32_t xa = blockIdx.x * (2 * blockDim.x) + warp * 64 + lane;
   if (xa >= g.nx) return;
   if constexpr (AHEAD)
-    prefetch_ahead<S>(src, g, (uint64_t)(blockIdx.z + g.zb) * g.nxy +
+    prefetch_ahead<S, MODE>(src, g, (uint64_t)(blockIdx.z + g.zb) * g.nxy +
                                   (uint64_t)blockIdx.y * g.nx + blockIdx.x * (2 * blockDim.x));
   const bool vb = xa + 32 < g.nx;
   const uint32_t z = blockIdx.z + g.zb;
@@ -159,7 +162,7 @@ __global__ void __launch_bounds__(128, 3) adj_step_kernel(const S* src, S* dst, 
                                                        StepCounters* ctr) {
   wait_before();
   if constexpr (AHEAD)
-    prefetch_ahead<S>(src, g, (uint64_t)(blockIdx.z + g.zb) * g.nxy +
+    prefetch_ahead<S, MODE>(src, g, (uint64_t)(blockIdx.z + g.zb) * g.nxy +
                                   (uint64_t)blockIdx.y * g.nx + 2 * blockIdx.x * blockDim.x);
   const uint32_t x = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
   if (x >= g.nx) return;
@@ -179,7 +182,7 @@ __global__ void __launch_bounds__(128, 3) adj_linear_kernel(const S* src, S* dst
   wait_before();
   const uint32_t n = g.zb * g.nxy + 2 * (blockIdx.x * blockDim.x + threadIdx.x);  // P < 2^31
   if (n >= g.ze * g.nxy) return;
-  if constexpr (AHEAD) prefetch_ahead<S>(src, g, n - 2 * threadIdx.x);
+  if constexpr (AHEAD) prefetch_ahead<S, MODE>(src, g, n - 2 * threadIdx.x);
   const uint32_t row = n / g.nx;
   const uint32_t z = row / g.ny;
   node_update_adj<S, MODE, RECORD>(src, dst, g, n - row * g.nx, row - z * g.ny, z, cp, gamma_out,
@@ -194,6 +197,10 @@ __global__ void __launch_bounds__(128, 3) adj_linear_kernel(const S* src, S* dst
 // Rule: up to 2^18 nodes. us a step with the pass -> without: FP32 pull 16^3 3.5 -> 2.6 (the rate at
 // which the host launches), 32^3 3.6 -> 2.7, 48^3 5.1 -> 4.2, 64^3 9.0 -> 8.3, AA 32^3 5.2 -> 3.2, 64^3
 // 9.6 -> 9.3; beyond, the call in the step kernel costs more than the pass (128^3 AA 69.8 -> 77.3).
+// That is with nothing flagged; with flagged nodes the pass, a few blocks on a small box, is the slower
+// one by more (pull, with the pass -> here): every node flagged (uniform flow) 32^3 375 -> 18, 64^3 398
+// -> 67 us a step; the first 20 steps of a Taylor-Green field 32^3 25.9 -> 4.8, 64^3 31 -> 12, of a Kida
+// field 27.3 -> 6.2, 34 -> 15.
 constexpr uint64_t kSmallNodes = 1ull << 18;
 template <int MODE>
 __device__ __noinline__ void recollide_here(const float* src, float* dst, Geo g, uint32_t n,
@@ -256,7 +263,7 @@ static cudaError_t launch_adj(const S* src, S* dst, const Geo& g, const CollideP
                             gamma_out, ctr);
   };
   if constexpr (sizeof(S) == 2 || MODE != MODE_PULL) {
-    if (beyond_l2<S>(g)) return run(std::true_type{});
+    if (beyond_l2<S, MODE>(g)) return run(std::true_type{});
   }
   return run(std::false_type{});
 }
@@ -274,7 +281,7 @@ __global__ void __launch_bounds__(128, 3) pair_linear_kernel(const S* src, S* ds
   const uint32_t nend = g.ze * g.nxy;  // P < 2^31
   const uint32_t n = g.zb * g.nxy + blockIdx.x * 256 + warp * 64 + lane;
   if (n >= nend) return;
-  if (beyond_l2<S>(g)) prefetch_ahead<S>(src, g, g.zb * g.nxy + blockIdx.x * 256);
+  if (beyond_l2<S, MODE>(g)) prefetch_ahead<S, MODE>(src, g, g.zb * g.nxy + blockIdx.x * 256);
   const uint32_t row = n / g.nx;
   const uint32_t xa = n - row * g.nx;
   const uint32_t za = row / g.ny;
@@ -322,11 +329,7 @@ static cudaError_t launch_pair(const S* src, S* dst, const Geo& g, const Collide
         pair_step_kernel<S, MODE, RECORD, CENTRAL, POLY, decltype(ahead)::value>, grid, 32 * warps,
         st, src, dst, g, cp, gamma_out, ctr);
   };
-  // FP32 pull: short rows only (central moments without -> with: 128^3 81.9 -> 75.3 us, 192^3
-  // 266 -> 259, but 256^3 607 -> 628, 384^3 2109 -> 2164), and without the code for it, which
-  // costs those 3 % even where it is not taken
-  if (beyond_l2<S>(g) && (sizeof(S) == 2 || MODE != MODE_PULL || g.nx < 256))
-    return run(std::true_type{});
+  if (beyond_l2<S, MODE>(g)) return run(std::true_type{});
   return run(std::false_type{});
 }
 
