@@ -67,8 +67,9 @@ enum {
  * gamma = 2). LB_GAMMA_EXACT runs in the one-node-per-thread direct kernel only and is not
  * available to batches. */
 enum { LB_GAMMA_ESTIMATE = 0, LB_GAMMA_LBGK = 1, LB_GAMMA_RLB = 2, LB_GAMMA_EXACT = 3 };
-/* Storage of the populations in device memory; collision arithmetic is FP64 for LB_F64 and
- * FP32 otherwise. All three store the shift f_i - W_i; LB_F16 stores (f_i - W_i)/W_i in
+/* Storage of the populations in device memory; collision arithmetic is FP64 for LB_F64 (or 64-bit
+ * fixed point of a unit that follows the node, whose error relative to the node's shifts is not
+ * above that of FP64 instructions at any amplitude) and FP32 otherwise. All three store the shift f_i - W_i; LB_F16 stores (f_i - W_i)/W_i in
  * IEEE half precision, rounded to nearest even. */
 enum { LB_F64 = 0, LB_F32 = 1, LB_F16 = 2 };
 /* Streaming: LB_PULL keeps two population arrays (gather, collide, write);

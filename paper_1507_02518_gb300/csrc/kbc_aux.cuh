@@ -48,10 +48,10 @@ __device__ __forceinline__ S* canon_ptr(S* buf, const Geo& g, const Nbr& nb) {
 // W. Values outside the normal ranges go to the compiler's conversions.
 
 // 256^3, FP32 pull, one thread per node (before: a grid-stride loop with the layout picked at run
-// time): get 1.83 -> 1.07 ms, set 1.65 -> 1.33, moments 4.05 -> 0.73, init 6.09 -> 1.01; their
+// time): get 1.83 -> 1.07 ms, set 1.65 -> 1.33, moments 4.05 -> 0.73, init 6.09 -> 0.77; their
 // traffic alone takes 0.81, 0.81, 0.35, 0.33 ms. FP16: get 1.77 -> 1.06, set 2.52 -> 1.11, moments
-// 4.06 -> 0.62, init 6.98 -> 1.08; FP64: get 1.29 -> 1.08, set 1.55 -> 1.11, moments 3.21 -> 0.76.
-// Moments and init are bound by the integer pipe (400 and 1250 instructions a node), get and set
+// 4.06 -> 0.62, init 6.98 -> 0.87; FP64: get 1.29 -> 1.08, set 1.55 -> 1.11, moments 3.21 -> 0.76.
+// Moments and init are bound by the integer pipe (moments: 400 instructions a node), get and set
 // by DRAM and the FP64 addition together.
 
 // FP32 to FP64 exactly for normal numbers; *odd is set for zero, subnormals, infinities and NaN
@@ -338,7 +338,7 @@ __device__ __noinline__ void init_node_small(S* buf, Geo g, uint32_t x, uint32_t
 // f = f_eq(rho, u). FP32 and FP16 storage: the equilibrium's moments and populations in fixed
 // point (kbc_fix.cuh; 2^-59 absolute, far below the rounding of the stored values), for nodes
 // whose velocity or density shift is at least 2^-18, so that this holds relative to the node too.
-// The integer pipe bounds it (73 % busy); the writes are 0.32 of the FP32 kernel's 0.80 ms at 256^3.
+// The integer pipe bounds it (73 % busy); the writes are 0.32 of the FP32 kernel's 0.77 ms at 256^3.
 template <typename S, int KIND>
 __global__ void __launch_bounds__(256) init_kernel(S* buf, Geo g, const double* rho,
                                                    const double* u, uint64_t n0, uint64_t cnt,

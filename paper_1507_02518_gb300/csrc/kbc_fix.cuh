@@ -247,7 +247,7 @@ template <int S> KBC_HD float window(fx v, uint32_t sticky) {
 // of bits 36 and above and of the 24 below, both exact in FP32, is rounded once; the last 12 bits
 // count as a sticky bit, two places below the rounding one. Less than that is normalised first
 // (that way for every value took 36 of the 57 instructions a population of an FP32
-// initialisation: 256^3 1.00 -> 0.80 ms).
+// initialisation: 256^3 1.00 -> 0.77 ms).
 KBC_HD bool short_way(fx v) { return (uint32_t)((int32_t)((uint64_t)v >> 32) + 64) >= 128u; }
 template <int N> KBC_HD float to_f32_short(fx v) {
   return add_rn<24 + N>((float)((int32_t)((uint64_t)v >> 32) >> 4),

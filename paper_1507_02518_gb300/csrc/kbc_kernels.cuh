@@ -368,7 +368,8 @@ __device__ __forceinline__ CollideParams box_cp(const BoxDesc& bd, int with_t, i
 }
 
 // Batched ensemble: a persistent grid walks the work list; item k covers rows
-// [row0, row0 + nrows) (row = y + ny z) of one box.
+// [row0, row0 + nrows) (row = y + ny z) of one box. (This kernel: FP64 storage, and one node per
+// thread; 24 FP64 boxes of 32^3 to 128^3, 14.3 ms a step in FP64 instructions, 3.74 in fixed point.)
 template <typename S, int MODE, bool RECORD, bool CENTRAL>
 __global__ void __launch_bounds__(MaxThreads<S>::value) batch_kernel(const BoxDesc* __restrict__ boxes,
                                                     const WorkItem* __restrict__ items,
@@ -470,8 +471,8 @@ constexpr int kPassBlocks = 152;   // one wave: the pass kernels run one block p
 // the flagged nodes among the mask words of warps w0, w0 + stride, ... (32 words a warp);
 // returns the guard events. A warp takes its words' flagged nodes 32 at a time in the node order,
 // a node per lane, so that runs of flagged nodes are read and written coalesced; a node per word
-// and thread (words in a loop over their bits) touched a sector per value and took 20 ms for a
-// full 256^3 box.
+// and thread (words in a loop over their bits) touched a sector per value: a full 256^3 box took
+// 20 ms, 4.2 now (3.7 with a fixed unit and products rounded down throughout, see kbc_fix.cuh).
 template <typename S, int MODE, bool CENTRAL, bool POLY>
 __device__ unsigned long long fp64_pass_words(const S* src, S* dst, const Geo& g,
                                               const CollideParams& cp,
