@@ -1377,15 +1377,17 @@ template <> struct Pattern<MODE_AA_ODD> {
 };
 
 // Where plane `plane` holds what node n loads from it, for every n that is not at an edge of the box in
-// x or y (x shifts left out): a node of the box for every n of the box.
-template <int MODE> __host__ __device__ inline uint64_t ahead_node(const Geo& g, uint32_t plane,
-                                                                   uint64_t n) {
+// x or y (x shifts left out): a node of the box for every n of the box. (32-bit arithmetic: a box
+// holds fewer than 2^31 nodes.)
+template <int MODE> __host__ __device__ inline uint32_t ahead_node(const Geo& g, uint32_t plane,
+                                                                   uint32_t n) {
   if (MODE == MODE_AA_EVEN) return n;
   // the plane's own velocity: a pull step loads plane i at -v_i, an odd AA step plane 26 - i there
-  const int y = (int)(plane / 3 % 3) - 1, z = (int)(plane / 9) - 1;
-  const int64_t o = y * (int64_t)g.nx + z * (int64_t)g.nxy;
-  const int64_t m = (int64_t)n + (MODE == MODE_PULL ? -o : o);
-  return (uint64_t)(m < 0 ? m + (int64_t)g.P : (m >= (int64_t)g.P ? m - (int64_t)g.P : m));
+  const uint32_t zp = plane / 9, yp = plane / 3 - 3 * zp;
+  const int y = (int)yp - 1, z = (int)zp - 1;
+  const int o = y * (int)g.nx + z * (int)g.nxy, s = MODE == MODE_PULL ? -o : o;
+  const uint32_t P = (uint32_t)g.P, m = n + (s < 0 ? P + (uint32_t)s : (uint32_t)s);  // below 2 P
+  return m >= P ? m - P : m;
 }
 
 // One node loaded, collided in FP64 instructions (collide<double>, with the oracle's guard) and

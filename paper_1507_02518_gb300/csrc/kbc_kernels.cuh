@@ -117,15 +117,15 @@ __device__ __forceinline__ void advance_node(uint32_t& x, uint32_t& y, uint32_t&
 // 438.)
 constexpr uint32_t kWave = 456;
 template <typename S, int MODE>
-__device__ __forceinline__ void prefetch_ahead(const S* src, const Geo& g, uint64_t n) {
+__device__ __forceinline__ void prefetch_ahead(const S* src, const Geo& g, uint32_t n) {
   const uint32_t lane = threadIdx.x & 31;
-  n += (uint64_t)kWave * 2 * blockDim.x + 2 * (threadIdx.x & ~31u);
-  if (lane < 27 && n < g.P) {
+  n += kWave * 2 * blockDim.x + 2 * (threadIdx.x & ~31u);
+  if (lane < 27 && n < (uint32_t)g.P) {
     n = ahead_node<MODE>(g, lane, n);
     const S* p = src + (uint64_t)lane * g.P + n;
     asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
     // FP32: the second half of the warp's 64 nodes
-    if (sizeof(S) == 4 && n + 32 < g.P) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + 32));
+    if (sizeof(S) == 4 && n + 32 < (uint32_t)g.P) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + 32));
   }
 }
 // where it is worth its instructions: a step's populations (pull: both buffers) larger than L2
@@ -145,8 +145,8 @@ __global__ void __launch_bounds__(128, 3) pair_step_kernel(const S* src, S* dst,
   const uint32_t xa = blockIdx.x * (2 * blockDim.x) + warp * 64 + lane;
   if (xa >= g.nx) return;
   if constexpr (AHEAD)
-    prefetch_ahead<S, MODE>(src, g, (uint64_t)(blockIdx.z + g.zb) * g.nxy +
-                                  (uint64_t)blockIdx.y * g.nx + blockIdx.x * (2 * blockDim.x));
+    prefetch_ahead<S, MODE>(src, g, (blockIdx.z + g.zb) * g.nxy + blockIdx.y * g.nx +
+                                        blockIdx.x * (2 * blockDim.x));
   const bool vb = xa + 32 < g.nx;
   const uint32_t z = blockIdx.z + g.zb;
   node_update2<S, MODE, RECORD, CENTRAL, POLY>(src, dst, g, xa, blockIdx.y, z,
@@ -162,8 +162,8 @@ __global__ void __launch_bounds__(128, 3) adj_step_kernel(const S* src, S* dst, 
                                                        StepCounters* ctr) {
   wait_before();
   if constexpr (AHEAD)
-    prefetch_ahead<S, MODE>(src, g, (uint64_t)(blockIdx.z + g.zb) * g.nxy +
-                                  (uint64_t)blockIdx.y * g.nx + 2 * blockIdx.x * blockDim.x);
+    prefetch_ahead<S, MODE>(src, g, (blockIdx.z + g.zb) * g.nxy + blockIdx.y * g.nx +
+                                        2 * blockIdx.x * blockDim.x);
   const uint32_t x = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
   if (x >= g.nx) return;
   node_update_adj<S, MODE, RECORD>(src, dst, g, x, blockIdx.y, blockIdx.z + g.zb, cp,

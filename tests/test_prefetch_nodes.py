@@ -33,8 +33,28 @@ template <int MODE> int check(uint32_t nx, uint32_t ny, uint32_t nz) {
   }
   return bad;
 }
+// the largest boxes: nodes near 2^31
+template <int MODE> int check_large(uint32_t nx, uint32_t ny, uint32_t nz) {
+  Geo g = {};
+  g.nx = nx, g.ny = ny, g.nz = nz, g.nxy = nx * ny, g.P = (uint64_t)nx * ny * nz;
+  int bad = 0;
+  for (uint32_t plane = 0; plane < 27; ++plane)
+    for (uint64_t k = 0; k < g.P; k += g.P / 1000 - 1) {
+      const int64_t o = ((int)(plane / 3 % 3) - 1) * (int64_t)nx + ((int)(plane / 9) - 1) * (int64_t)g.nxy;
+      for (uint64_t n : {k, g.P - 1 - k}) {
+        int64_t m = (int64_t)n + (MODE == MODE_PULL ? -o : MODE == MODE_AA_ODD ? o : 0);
+        m = (m + (int64_t)g.P) % (int64_t)g.P;
+        bad += ahead_node<MODE>(g, plane, (uint32_t)n) != (uint64_t)m;
+      }
+    }
+  return bad;
+}
 int main() {
   int bad = 0;
+  const uint32_t l[3][3] = {{1290, 1290, 1290}, {26754, 26754, 3}, {3, 3, 238609294}};
+  for (auto& b : l)
+    bad += check_large<MODE_PULL>(b[0], b[1], b[2]) + check_large<MODE_AA_EVEN>(b[0], b[1], b[2]) +
+           check_large<MODE_AA_ODD>(b[0], b[1], b[2]);
   const uint32_t s[5][3] = {{3, 3, 3}, {8, 5, 4}, {7, 3, 9}, {64, 6, 3}, {5, 16, 7}};
   for (auto& b : s)
     bad += check<MODE_PULL>(b[0], b[1], b[2]) + check<MODE_AA_EVEN>(b[0], b[1], b[2]) +
