@@ -22,12 +22,12 @@
 //   * the entropic products, of which a ratio is taken, are integer products too, of deviations
 //     scaled by a common power of two to about 2^59, with integer weights that need no
 //     reciprocal.
-// About 3500 instructions per node, of which 54 (the conversions of the changes and the additions)
+// About 4000 instructions per node, of which 54 (the conversions of the changes and the additions)
 // are the FP64 pipe's, which they fill for nearly half of the time; 16 warps per SM.
-// Measured at 256^3 (FP64 pull): FP64 instructions 17.4 ms a step, this 3.2 ms; 432 B a node take
+// Measured at 256^3 (FP64 pull): FP64 instructions 17.4 ms a step, this 3.27; 432 B a node take
 // 1.08 ms. A fixed unit of 2^-60, without the change and with products rounded down took 2.85 ms (32^3
-// 8.7 us, now 11.3) but lost momentum one-sidedly, and small shifts their bits. The sum in integers
-// instead of FP64: 3.48 ms.
+// 8.7 us, now 11.3) but lost momentum one-sidedly, and small shifts their bits. With the last sum
+// in integers instead of FP64 a step is 9 % slower.
 // Nodes outside the range of the format (|f - W| >= 1/4 or all below 2^-70, rho or u far from a
 // lattice state, NaN, |beta gamma| >= 128) are reported and left to the FP64 collision.
 //
@@ -312,7 +312,7 @@ KBC_HD fx mul(Split a, Split b) {
 }
 // The same with each cross term rounded down, a unit low on average unless a factor is 0: two high
 // halves instead of two wide multiplies, which take twice as long (256^3 FP64 pull with every product
-// to nearest 3.45 ms, with the 81 innermost entropic ones by this 3.2). For sums that start with
+// to nearest is 8 % slower than with the 81 innermost entropic ones by this). For sums that start with
 // what they will lose.
 KBC_HD fx mul_down(Split a, Split b) {
   return (long long)a.h * b.h + (mul_high(a.h, b.l) + mul_high(a.l, b.h));

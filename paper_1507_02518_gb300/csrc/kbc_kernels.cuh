@@ -69,10 +69,10 @@ __global__ void __launch_bounds__(MaxThreads<S>::value) step_kernel(const S* src
 }
 
 // The FP64 step with the fixed-point collision, one node per thread over the node order, so that
-// rows of any length keep every lane busy (the two divisions are nothing beside the ~3400
+// rows of any length keep every lane busy (the two divisions are nothing beside the ~4000
 // instructions of the collision): with 128-thread rows 22 % of a 100^3 box's lanes idled. 128
-// registers give 16 warps per SM: 256^3 pull 3.20 ms, 3.58 at 168 (12 warps), 3.31 at 112; 100^3 AA
-// 196, 218, 204 us; 32^3 pull 11.3, 11.0, 11.7.
+// registers give 16 warps per SM: 256^3 pull 3.20 ms, 3.58 at 168 (12 warps), 3.31 at 112 (all in one
+// session; 3.27 in others); 100^3 AA 196, 218, 204 us; 32^3 pull 11.3, 11.0, 11.7.
 template <int MODE, bool RECORD>
 __global__ void __maxnreg__(128) fix_step_kernel(const double* src, double* dst, Geo g,
                                                          CollideParams cp, float* gamma_out,
